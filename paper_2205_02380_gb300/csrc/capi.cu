@@ -709,7 +709,7 @@ size_t chasm_workspace_bytes(const chasm_grid* grid, const chasm_potential* pot,
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) sms = 152;
     ThetaPlan tp;
     if (xs) {
-      w += xs_table_bytes(nk, nxp, e);
+      w += xs_alloc_bytes(nk, nxp, e);
       theta_xs_plan(nk, fp64, nxp, sms, &tp);
     } else {
       w += 2 * fbytes;
@@ -814,7 +814,7 @@ int chasm_create(const chasm_grid* grid, const chasm_box* box, const chasm_poten
     if (e != cudaSuccess) return bail(cuda_fail(H, e, "symbol precompute"));
     H->xs = table_form(N, g.nxp, H->elt, o);
     if (H->xs) {
-      if (cudaMallocAsync(&H->d_sig, xs_table_bytes(N, g.nxp, H->elt), H->stream) != cudaSuccess)
+      if (cudaMallocAsync(&H->d_sig, xs_alloc_bytes(N, g.nxp, H->elt), H->stream) != cudaSuccess)
         return bail(fail(H, CHASM_ENOMEM, "device allocation failed (per-x symbol table)"));
       e = build_xs_table(*H, H->d_sig, H->stream);
       if (e != cudaSuccess) return bail(cuda_fail(H, e, "per-x symbol table"));
@@ -967,7 +967,7 @@ int chasm_tkm_convolve(chasm_handle* h, const void* g, void* phi) {
     return fail(H, CHASM_EINVAL, "g/phi must be 16-byte aligned");
   if (!H->d_tkm) {   // the spectrum of T, built once per handle on first use
     const int N = H->g.nk;
-    const size_t bytes = (size_t)4 * N * N * N * H->elt;
+    const size_t bytes = xs_alloc_bytes(N, 1, H->elt);
     if (cudaMallocAsync(&H->d_tkm, bytes, H->stream) != cudaSuccess) {
       H->d_tkm = nullptr;
       return fail(H, CHASM_ENOMEM, "chasm_tkm_convolve: table allocation failed");

@@ -1,0 +1,226 @@
+// Register-resident FFTs on block fixed-point data: the FP64-class arithmetic of the table-form
+// P(dt) kernel (k_theta_fx.cu).
+//
+// Why.  GB300 issues 1.7 FP64 FMAs per clock and SM (measured) against 60 64-bit integer adds and
+// 24 wide integer multiply-adds.  A vector that one thread transforms is therefore held as 64-bit
+// integers with one common binary exponent:
+//   value_n = x_n 2^E,   |Re x_n|, |Im x_n| <= 2^57 on entry of a transform of length <= 32,
+// so that the largest output of the transform (modulus <= 32 * 2^57.5) still fits.  Additions are
+// exact; a product with a twiddle constant of 64 fractional bits is off by at most two units of
+// 2^E, i.e. 2^-56 of the vector's largest entry, where an FP64 FMA rounds at 2^-53 of each
+// result.  Between transforms a vector keeps its exponent and the number of magnitude bits it
+// uses, and the next transform aligns what it gathers to 57 bits again.
+//
+// A rotation by an angle up to 45 degrees is done by three lifting steps
+//   x += a y, y += s x, x += a y,  a = -tan(phi/2), s = sin(phi)
+// (Daubechies and Sweldens, "Factoring wavelet transforms into lifting steps", J. Fourier Anal.
+// Appl. 1998, apply the factorisation to rotations): three products instead of four, and every
+// constant stays below one half after 1 - s replaces an s above it.
+#pragma once
+
+#include <cstdint>
+#include <type_traits>
+
+namespace chasm {
+namespace {
+
+using i64 = long long;
+using u64 = unsigned long long;
+
+// ---- constants with 64 fractional bits, evaluated at compile time ----
+using fx128 = unsigned __int128;
+constexpr u64 kFxPi61 = 0x6487ED5110B4611AULL;   // pi 2^61 (pi = 3.243F6A88 85A308D3 ... hex)
+constexpr u64 fx_mulq(u64 a, u64 b) { return (u64)(((fx128)a * b) >> 64); }
+constexpr u64 fx_divq(u64 a, u64 b) {   // a / b with 64 fractional bits, a < b
+  return (u64)((((fx128)a) << 64) / b);
+}
+// 2 pi k / m for 0 < k / m <= 1/8, 64 fractional bits (at most pi / 4 < 1)
+constexpr u64 fx_angle(int k, int m) { return (u64)((((fx128)kFxPi61) * 16 * (unsigned)k) / (unsigned)m); }
+constexpr u64 fx_sin_series(u64 x) {
+  const u64 x2 = fx_mulq(x, x);
+  u64 t = x, s = x;
+  for (int i = 1; i < 14; ++i) {
+    t = fx_mulq(t, x2) / (unsigned)((2 * i) * (2 * i + 1));
+    s = (i & 1) ? s - t : s + t;
+  }
+  return s;
+}
+constexpr u64 fx_vers_series(u64 x) {   // 1 - cos x
+  const u64 x2 = fx_mulq(x, x);
+  u64 t = x2 / 2, s = t;
+  for (int i = 2; i < 14; ++i) {
+    t = fx_mulq(t, x2) / (unsigned)((2 * i - 1) * (2 * i));
+    s = (i & 1) ? s + t : s - t;
+  }
+  return s;
+}
+constexpr u64 fx_sin(int k, int m) { return fx_sin_series(fx_angle(k, m)); }
+constexpr u64 fx_vers(int k, int m) { return fx_vers_series(fx_angle(k, m)); }
+// sin, 1 - cos and tan(phi / 2) of phi = 2 pi K / M, 0 < K / M <= 1/8
+template <int K, int M>
+struct FxK {
+  static constexpr u64 sin = fx_sin(K, M);
+  static constexpr u64 vers = fx_vers(K, M);
+  static constexpr u64 cos = (u64)0 - vers;
+  static constexpr u64 tanh = fx_divq(fx_vers(K, M), fx_sin(K, M));
+};
+
+template <int B, int E, int S = 1, class F>
+__device__ __forceinline__ void xfor(F&& f) {
+  if constexpr (B < E) {
+    f(std::integral_constant<int, B>{});
+    xfor<B + S, E, S>(f);
+  }
+}
+
+// ---- products ----
+// x w for a constant w = C / 2^64 < 1/2, rounded down to within two units.  The constant's low
+// word is taken as signed, so both cross terms are single high products.
+template <u64 C>
+__device__ __forceinline__ i64 fx_mulc(i64 x) {
+  static_assert(C < (1ULL << 63) - (1ULL << 32), "constants below one half");
+  constexpr int wl = (int)(unsigned)C;
+  constexpr unsigned wh = (unsigned)((C >> 32) + (((unsigned)C) >> 31));
+  const int xh = (int)(x >> 32);
+  const unsigned xl = (unsigned)x;
+  const i64 r = (i64)(int)wh * (i64)xh + (i64)(u64)__umulhi(wh, xl);
+  return r + (i64)__mulhi(wl, xh);
+}
+// a +- x w, 0 <= w <= 1 given as C / 2^64
+template <bool NEG, u64 C>
+__device__ __forceinline__ i64 fx_fma(i64 a, i64 x) {
+  if constexpr (C < (1ULL << 63) - (1ULL << 32)) {
+    const i64 p = fx_mulc<C>(x);
+    return NEG ? a - p : a + p;
+  } else {   // x w = x - x (1 - w)
+    const i64 p = fx_mulc<(u64)0 - C>(x);
+    return NEG ? (a - x) + p : (a + x) - p;
+  }
+}
+// x w
+template <u64 C>
+__device__ __forceinline__ i64 fx_mul(i64 x) {
+  if constexpr (C < (1ULL << 63) - (1ULL << 32)) return fx_mulc<C>(x);
+  else return x - fx_mulc<(u64)0 - C>(x);
+}
+struct fxc {
+  i64 re, im;
+};
+
+// z e^{-2 pi i K / M} (INV: e^{+2 pi i K / M}), 8 | M
+template <int K_, int M, bool INV>
+__device__ __forceinline__ fxc fx_rot(fxc z) {
+  constexpr int K = ((INV ? K_ : -K_) % M + M) % M;   // by the angle +2 pi K / M
+  constexpr int q = (K + M / 8 - 1) / (M / 4);        // quarter turns taken out: rest in (-M/8, M/8]
+  constexpr int r = K - q * (M / 4);
+  constexpr int a = r < 0 ? -r : r;
+  if constexpr (8 * a == M) {          // 45 degrees: (x -+ y) / sqrt 2, 1 / sqrt 2 = 1 - vers
+    constexpr u64 V = FxK<1, 8>::vers;
+    const i64 d = r > 0 ? z.re - z.im : z.re + z.im;
+    const i64 s = r > 0 ? z.re + z.im : z.im - z.re;
+    z = {d - fx_mulc<V>(d), s - fx_mulc<V>(s)};
+  } else if constexpr (a != 0) {
+    constexpr u64 T = FxK<a, M>::tanh, S = FxK<a, M>::sin;
+    z.re = fx_fma<(r > 0), T>(z.re, z.im);
+    z.im = fx_fma<(r < 0), S>(z.im, z.re);
+    z.re = fx_fma<(r > 0), T>(z.re, z.im);
+  }
+  if constexpr ((q & 3) == 1) return {-z.im, z.re};
+  else if constexpr ((q & 3) == 2) return {-z.re, -z.im};
+  else if constexpr ((q & 3) == 3) return {z.im, -z.re};
+  else return z;
+}
+
+// ---- transforms ----
+// DFT_4 in place, natural order: X_j = sum_n x_n e^{-2 pi i jn/4}
+__device__ __forceinline__ void fx_dft4(fxc& a, fxc& b, fxc& c, fxc& d) {
+  const fxc s = {a.re + c.re, a.im + c.im}, t = {a.re - c.re, a.im - c.im};
+  const fxc u = {b.re + d.re, b.im + d.im}, v = {b.re - d.re, b.im - d.im};
+  a = {s.re + u.re, s.im + u.im};
+  b = {t.re + v.im, t.im - v.re};
+  c = {s.re - u.re, s.im - u.im};
+  d = {t.re - v.im, t.im + v.re};
+}
+
+// DFT_M (M = 4, 8, 16) of x[0..M), natural order in and out, by radix 4: 4 rotations by 45 degrees
+// and 4 others at M = 16 (radix 2: 6 and 4)
+template <int M>
+__device__ __forceinline__ void fx_dft(fxc* x) {
+  static_assert(M == 4 || M == 8 || M == 16, "DFT lengths");
+  if constexpr (M == 4) {
+    fx_dft4(x[0], x[1], x[2], x[3]);
+  } else {
+    constexpr int R = M / 4;   // M = 4 R: DFT_4 over n = i + R m, twiddle, DFT_R over i
+    xfor<0, R>([&](auto I) {
+      constexpr int i = decltype(I)::value;
+      fx_dft4(x[i], x[i + R], x[i + 2 * R], x[i + 3 * R]);   // x[i + R k2]
+      xfor<1, 4>([&](auto K) {
+        constexpr int k2 = decltype(K)::value;
+        x[i + R * k2] = fx_rot<i * k2, M, false>(x[i + R * k2]);
+      });
+    });
+    fxc y[M];
+    xfor<0, 4>([&](auto K) {
+      constexpr int k2 = decltype(K)::value;
+      if constexpr (R == 4) {
+        fx_dft4(x[4 * k2], x[4 * k2 + 1], x[4 * k2 + 2], x[4 * k2 + 3]);
+        xfor<0, 4>([&](auto J) { y[k2 + 4 * decltype(J)::value] = x[4 * k2 + decltype(J)::value]; });
+      } else {
+        const fxc a = x[2 * k2], b = x[2 * k2 + 1];
+        y[k2] = {a.re + b.re, a.im + b.im};
+        y[k2 + 4] = {a.re - b.re, a.im - b.im};
+      }
+    });
+    xfor<0, M>([&](auto J) { x[decltype(J)::value] = y[decltype(J)::value]; });
+  }
+}
+
+// A transform of length N (8, 16, 32) is two of length N / 2 (fft_fx_core) and one radix-2 step
+// before it (fft_fx_pre: x in time order) or after it (fft_fx_post: x out in time order); the
+// frequencies sit at x[j] = X_{fx_freq(j)}, the even ones first.  ODD: the odd outputs of a
+// zero-padded length-2N transform, X_q = sum_n x_n e^{-2 pi i (2q + 1) n / (2N)}, or the sum over
+// such frequencies: its radix-2 step holds the twist e^{-i pi n / N} in its own rotations.  All
+// transforms have the sign of e^{-i...}; the other sign is this one on (im, re).
+// On entry |Re|, |Im| <= 2^57 (N = 32); the outputs stay below 2^63.
+template <int N>
+__host__ __device__ constexpr int fx_freq(int j) { return 2 * (j % (N / 2)) + j / (N / 2); }
+
+template <int N, bool ODD>
+__device__ __forceinline__ void fft_fx_pre(fxc (&x)[N]) {
+  constexpr int M = N / 2;
+  xfor<0, M>([&](auto I) {
+    constexpr int n = decltype(I)::value;
+    const fxc a = x[n], b = x[n + M];
+    if constexpr (ODD) {
+      x[n] = fx_rot<n, 2 * N, false>(fxc{a.re + b.im, a.im - b.re});            // a - i b
+      x[n + M] = fx_rot<3 * n, 2 * N, false>(fxc{a.re - b.im, a.im + b.re});    // a + i b
+    } else {
+      x[n] = {a.re + b.re, a.im + b.im};
+      x[n + M] = fx_rot<n, N, false>(fxc{a.re - b.re, a.im - b.im});
+    }
+  });
+}
+template <int N>
+__device__ __forceinline__ void fft_fx_core(fxc (&x)[N]) {
+  fx_dft<N / 2>(x);
+  fx_dft<N / 2>(x + N / 2);
+}
+template <int N, bool ODD>
+__device__ __forceinline__ void fft_fx_post(fxc (&x)[N]) {
+  constexpr int M = N / 2;
+  xfor<0, M>([&](auto I) {
+    constexpr int n = decltype(I)::value;
+    if constexpr (ODD) {
+      const fxc a = fx_rot<n, 2 * N, false>(x[n]), b = fx_rot<3 * n, 2 * N, false>(x[n + M]);
+      x[n] = {a.re + b.re, a.im + b.im};
+      x[n + M] = {a.im - b.im, b.re - a.re};   // -i (a - b)
+    } else {
+      const fxc a = x[n], b = fx_rot<n, N, false>(x[n + M]);
+      x[n] = {a.re + b.re, a.im + b.im};
+      x[n + M] = {a.re - b.re, a.im - b.im};
+    }
+  });
+}
+
+}  // namespace
+}  // namespace chasm

@@ -257,11 +257,6 @@ __device__ __forceinline__ float ld_stream(const float* p, uint64_t pol) {
   asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
   return v;
 }
-__device__ __forceinline__ double ld_stream(const double* p, uint64_t pol) {
-  double v;
-  asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v) : "l"(p), "l"(pol));
-  return v;
-}
 
 // two adjacent single-precision complex values per access (16-byte aligned)
 __device__ __forceinline__ void ld2_keep(const cpx<float>* p, uint64_t pol, cpx<float>& a, cpx<float>& b) {
@@ -410,7 +405,9 @@ __device__ __forceinline__ void slab_conv(cpx<T>* Gs, cpx<T>* V, const T* __rest
     if constexpr (IMAG) spol = l2_stream_policy();
 #pragma unroll
     for (int j = 0; j < N; ++j) {
-      const T w = IMAG ? ld_stream(t + (size_t)j * L, spol) : __ldg(t + (size_t)j * L);
+      T w;
+      if constexpr (IMAG) w = ld_stream(t + (size_t)j * L, spol);
+      else w = __ldg(t + (size_t)j * L);
       if constexpr (IMAG) {
         const T a = re[j];
         re[j] = -w * im[j];

@@ -100,6 +100,8 @@ cudaError_t measure_fma_peak_f32x2(double* tflops);
 cudaError_t measure_fft_pk_rate(double* tflops);
 // the per-x symbol table (k_xsym.cu), [nxp][N][2N][2N] in the storage type; needs H.d_T
 size_t xs_table_bytes(int nk, int64_t nxp, size_t elt);
+// bytes of its allocation: in double precision the column exponents follow the table
+size_t xs_alloc_bytes(int nk, int64_t nxp, size_t elt);
 cudaError_t build_xs_table(const Handle& H, void* sig, cudaStream_t s);
 // the spectrum of T on the same frequencies, (2 / (2N)^3) sum_m T_m e^{-i omega . m} (real: T is
 // even), one x point's worth of table in the layout of the per-x table; needs H.d_T
@@ -112,6 +114,15 @@ __host__ __device__ constexpr bool xs_packed(bool fp64, int nk) { return !fp64 &
 void theta_pk_plan(int nk, int64_t nxp, int num_sms, ThetaPlan* plan);
 cudaError_t launch_theta_pk(const Handle& H, const void* in, const void* base, void* out, int nst,
                             const double* coef, cudaStream_t s, const XsExtra& x);
+
+// Double precision (k_theta_fx.cu): block fixed-point arithmetic.  Its symbol table is the FP64
+// table of nxp x points converted in place by fx_symbol, followed by fx_symbol_extra_bytes of
+// column exponents.
+void theta_fx_plan(int nk, int64_t nxp, int num_sms, ThetaPlan* plan);
+cudaError_t launch_theta_fx(const Handle& H, const void* in, const void* base, void* out, int nst,
+                            const double* coef, cudaStream_t s, const XsExtra& x);
+size_t fx_symbol_extra_bytes(int nk, int64_t nxp);
+cudaError_t fx_symbol(void* sig, int nk, int64_t nxp, cudaStream_t s);
 
 constexpr size_t kXsAutoMaxBytes = (size_t)64 << 30;
 

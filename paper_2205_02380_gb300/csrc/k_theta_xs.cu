@@ -1,5 +1,6 @@
-// Coulomb operator and P-flow in the real form with a per-x symbol table (Sec. 4): FP64 and
-// N_k = 8 (single precision with N_k = 16 or 32 runs the packed kernel of k_theta_pk.cu).
+// Coulomb operator and P-flow in the real form with a per-x symbol table (Sec. 4): single
+// precision with N_k = 8 (N_k = 16 and 32 run the packed kernel of k_theta_pk.cu, double precision
+// the block fixed-point kernel of k_theta_fx.cu), and the dispatch over the three.
 //
 // For one x point, Theta^T is a real linear convolution over the k-grid:
 //   Theta^T[u]_p = sum_q S_{p-q}(x) u_q,
@@ -54,9 +55,10 @@ struct XsParams {
 // launch shape per (precision, N): threads, spectrum in shared memory, CTAs per SM compiled for
 template <typename T, int N>
 struct XsCfg {
-  static constexpr int NT = N == 32 ? (sizeof(T) == 4 ? 512 : 256) : (N == 16 ? 256 : 128);
-  static constexpr bool GSM = N <= 16;
-  static constexpr int MINB = (sizeof(T) == 4 && N == 16) ? 2 : 1;
+  static_assert(sizeof(T) == 4 && N == 8, "single precision, N_k = 8");
+  static constexpr int NT = 128;
+  static constexpr bool GSM = true;
+  static constexpr int MINB = 1;
   static constexpr int L = 2 * N;
   static constexpr int GS = 2 * N;
   static constexpr int NG = NT / GS;
@@ -110,79 +112,43 @@ __device__ __forceinline__ void load_col(const cpx<T>* g, int stride, T (&re)[N]
 template <typename T, int N>
 __device__ __forceinline__ void horner_line(T (&re)[N], const T (&im)[N], const T* b, const T* b2,
                                             T cb2, T c) {
-  if constexpr (sizeof(T) == 4 && N % 4 == 0) {
-    const float4* b4 = reinterpret_cast<const float4*>(b);
-    const float4* c4 = reinterpret_cast<const float4*>(b2);
+  const float4* b4 = reinterpret_cast<const float4*>(b);
+  const float4* c4 = reinterpret_cast<const float4*>(b2);
 #pragma unroll
-    for (int q = 0; q < N / 4; ++q) {
-      float4 bb = b ? b4[q] : make_float4(0.f, 0.f, 0.f, 0.f);
-      if (b2) {
-        const float4 cc = c4[q];
-        bb = make_float4(fmaf(cb2, cc.x, bb.x), fmaf(cb2, cc.y, bb.y), fmaf(cb2, cc.z, bb.z),
-                         fmaf(cb2, cc.w, bb.w));
-      }
-      const float bv[4] = {bb.x, bb.y, bb.z, bb.w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int n = 4 * q + e;
-        const T th = re[n] * ht_cos<T>(n * (32 / N)) - im[n] * ht_sin<T>(n * (32 / N));
-        re[n] = fma(c, th, (T)bv[e]);
-      }
+  for (int q = 0; q < N / 4; ++q) {
+    float4 bb = b ? b4[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (b2) {
+      const float4 cc = c4[q];
+      bb = make_float4(fmaf(cb2, cc.x, bb.x), fmaf(cb2, cc.y, bb.y), fmaf(cb2, cc.z, bb.z),
+                       fmaf(cb2, cc.w, bb.w));
     }
-  } else {
-    const double2* bd = reinterpret_cast<const double2*>(b);
-    const double2* cd = reinterpret_cast<const double2*>(b2);
+    const float bv[4] = {bb.x, bb.y, bb.z, bb.w};
 #pragma unroll
-    for (int q = 0; q < N / 2; ++q) {
-      double2 bb = b ? bd[q] : make_double2(0.0, 0.0);
-      if (b2) {
-        const double2 cc = cd[q];
-        bb = make_double2(fma((double)cb2, cc.x, bb.x), fma((double)cb2, cc.y, bb.y));
-      }
-      const T bv[2] = {(T)bb.x, (T)bb.y};
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int n = 2 * q + e;
-        const T th = re[n] * ht_cos<T>(n * (32 / N)) - im[n] * ht_sin<T>(n * (32 / N));
-        re[n] = fma(c, th, bv[e]);
-      }
+    for (int e = 0; e < 4; ++e) {
+      const int n = 4 * q + e;
+      const T th = re[n] * ht_cos<T>(n * (32 / N)) - im[n] * ht_sin<T>(n * (32 / N));
+      re[n] = fma(c, th, (T)bv[e]);
     }
   }
 }
 
 template <typename T, int N>
 __device__ __forceinline__ void store_line_cs(T* __restrict__ dst, const T (&v)[N]) {
-  if constexpr (sizeof(T) == 4 && N % 4 == 0) {
-    float4* d4 = reinterpret_cast<float4*>(dst);
+  float4* d4 = reinterpret_cast<float4*>(dst);
 #pragma unroll
-    for (int q = 0; q < N / 4; ++q) __stcs(d4 + q, make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
-  } else {
-    double2* d2 = reinterpret_cast<double2*>(dst);
-#pragma unroll
-    for (int q = 0; q < N / 2; ++q) __stcs(d2 + q, make_double2(v[2 * q], v[2 * q + 1]));
-  }
+  for (int q = 0; q < N / 4; ++q) __stcs(d4 + q, make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
 }
 
 template <typename T, int N>
 __device__ __forceinline__ void load_line_plain(const T* src, T (&v)[N]) {
-  if constexpr (sizeof(T) == 4 && N % 4 == 0) {
-    const float4* s4 = reinterpret_cast<const float4*>(src);
+  const float4* s4 = reinterpret_cast<const float4*>(src);
 #pragma unroll
-    for (int q = 0; q < N / 4; ++q) {
-      const float4 t = s4[q];
-      v[4 * q] = t.x;
-      v[4 * q + 1] = t.y;
-      v[4 * q + 2] = t.z;
-      v[4 * q + 3] = t.w;
-    }
-  } else {
-    const double2* s2 = reinterpret_cast<const double2*>(src);
-#pragma unroll
-    for (int q = 0; q < N / 2; ++q) {
-      const double2 t = s2[q];
-      v[2 * q] = (T)t.x;
-      v[2 * q + 1] = (T)t.y;
-    }
+  for (int q = 0; q < N / 4; ++q) {
+    const float4 t = s4[q];
+    v[4 * q] = t.x;
+    v[4 * q + 1] = t.y;
+    v[4 * q + 2] = t.z;
+    v[4 * q + 3] = t.w;
   }
 }
 
@@ -323,38 +289,15 @@ cudaError_t launch_xs_tn(const Handle& H, const void* in, const void* base, void
 cudaError_t launch_theta_xs(const Handle& H, const void* in, const void* base, void* out, int nst,
                             const double* coef, cudaStream_t s, const XsExtra& x) {
   if (nst < 1 || nst > 4 || !H.d_sig) return cudaErrorInvalidValue;
+  if (H.fp64) return launch_theta_fx(H, in, base, out, nst, coef, s, x);
   if (xs_packed(H.fp64, H.g.nk)) return launch_theta_pk(H, in, base, out, nst, coef, s, x);
-  switch (H.g.nk) {
-    case 8:
-      return H.fp64 ? launch_xs_tn<double, 8>(H, in, base, out, nst, coef, x, s)
-                    : launch_xs_tn<float, 8>(H, in, base, out, nst, coef, x, s);
-    case 16:
-      return H.fp64 ? launch_xs_tn<double, 16>(H, in, base, out, nst, coef, x, s) : cudaErrorInvalidValue;
-    case 32:
-      return H.fp64 ? launch_xs_tn<double, 32>(H, in, base, out, nst, coef, x, s) : cudaErrorInvalidValue;
-  }
-  return cudaErrorInvalidValue;
+  return launch_xs_tn<float, 8>(H, in, base, out, nst, coef, x, s);
 }
 
 void theta_xs_plan(int nk, bool fp64, int64_t nxp, int num_sms, ThetaPlan* pl) {
-  if (xs_packed(fp64, nk)) {
-    theta_pk_plan(nk, nxp, num_sms, pl);
-    return;
-  }
-  switch (nk) {
-    case 8:
-      fp64 ? plan_xs_tn<double, 8>(nxp, num_sms, pl) : plan_xs_tn<float, 8>(nxp, num_sms, pl);
-      return;
-    case 16:
-      if (fp64) plan_xs_tn<double, 16>(nxp, num_sms, pl);
-      return;
-    case 32:
-      if (fp64) plan_xs_tn<double, 32>(nxp, num_sms, pl);
-      return;
-  }
-  pl->cluster = 0;
-  pl->blocks = 1;
-  pl->scratch_bytes = 0;
+  if (fp64) theta_fx_plan(nk, nxp, num_sms, pl);
+  else if (xs_packed(fp64, nk)) theta_pk_plan(nk, nxp, num_sms, pl);
+  else plan_xs_tn<float, 8>(nxp, num_sms, pl);
 }
 
 }  // namespace chasm

@@ -239,6 +239,10 @@ cudaError_t run_table(const XsGeom& G, bool fp64, const double* Tfull, void* sig
 
 size_t xs_table_bytes(int nk, int64_t nxp, size_t elt) { return (size_t)nxp * 4 * nk * nk * nk * elt; }
 
+size_t xs_alloc_bytes(int nk, int64_t nxp, size_t elt) {
+  return xs_table_bytes(nk, nxp, elt) + (elt == 8 ? fx_symbol_extra_bytes(nk, nxp) : 0);
+}
+
 cudaError_t build_xs_table(const Handle& H, void* sig, cudaStream_t s) {
   XsGeom G{};
   const int N = H.g.nk, L = 2 * N;
@@ -256,7 +260,8 @@ cudaError_t build_xs_table(const Handle& H, void* sig, cudaStream_t s) {
     for (int d = 0; d < 3; ++d) G.pos[a][d] = H.nuclei[a].pos[d];
     G.g[a] = 2.0 * H.nuclei[a].charge / (M_PI * M_PI * H.hbar * (double)L * L * L);
   }
-  return run_table(G, H.fp64, H.d_T, sig, s);
+  const cudaError_t e = run_table(G, H.fp64, H.d_T, sig, s);
+  return e == cudaSuccess && H.fp64 ? fx_symbol(sig, N, H.g.nxp, s) : e;
 }
 
 // One x point at the (virtual) nucleus (a = 0), only the sg = 0 terms: sum_m T_m prod_d w(m_d)
@@ -277,7 +282,8 @@ cudaError_t build_tkm_table(const Handle& H, void* out, cudaStream_t s) {
   G.g[0] = 2.0 / ((double)L * L * L);
   G.plain = 1;
   if (!H.d_T) return cudaErrorInvalidValue;
-  return run_table(G, H.fp64, H.d_T, out, s);
+  const cudaError_t e = run_table(G, H.fp64, H.d_T, out, s);
+  return e == cudaSuccess && H.fp64 ? fx_symbol(out, N, 1, s) : e;
 }
 
 }  // namespace chasm
