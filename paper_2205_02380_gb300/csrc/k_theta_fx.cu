@@ -13,8 +13,8 @@
 // form needs about 3e7 operations of the 60-per-clock integer pipe (a 32-point transform takes 20
 // clocks per thread and SM against 231) and runs at about 60 % of that pipe, waiting for the
 // L2-resident spectrum, the symbol and the slab buffers with two warps per scheduler (64-bit
-// vectors of 32 complex values leave no registers for more).  P(dt): 224.3 -> 48.4 ms at
-// 16^3 x 32^3, 77.7 -> 13.9 ms at 24^3 x 16^3.
+// vectors of 32 complex values leave no registers for more).  P(dt): 224.3 -> 43.5 ms at
+// 16^3 x 32^3, 77.7 -> 13.4 ms at 24^3 x 16^3.
 //
 // Errors.  A vector enters a transform with 57 bits below its largest entry and leaves it with an
 // error of about 3 units of the last of them, so each of the eight transforms of a stage adds
@@ -77,8 +77,8 @@ struct FxCfg {
   static constexpr int TROW = N / 2 + 1;             // line staging row, 16-byte units
   static constexpr size_t v_bytes = (size_t)NG * VSZ * sizeof(fxc);
   static constexpr size_t g_bytes = GSM ? (size_t)N * N * N * sizeof(fxc) : 0;
-  // exA, exG [N][N]; ex1, ex2 [NG][64]; exP [NG][64]; etA, etG [N]; flag
-  static constexpr size_t e_bytes = (2 * N * N + 2 * NG * 64) * sizeof(int2) + (NG * 64 + 2 * N + 4) * sizeof(int);
+  // exA, exG [N][N]; ex1, ex2 [NG][64]; exP [NG][64]; etA, etG [N]; flag; three barriers per group
+  static constexpr size_t e_bytes = (2 * N * N + 2 * NG * 64) * sizeof(int2) + (NG * 64 + 2 * N + 4) * sizeof(int) + NG * 24;
   static constexpr size_t smem_bytes = v_bytes + g_bytes + e_bytes;
   static_assert(NG * VSZ * sizeof(fxc) / NW >= 32 * TROW * 16, "line staging fits the slab buffers");
 };
@@ -87,8 +87,28 @@ struct FxCfg {
 // two inverse halves are added: one bit less)
 constexpr int kFxBits = 57;
 
-__device__ __forceinline__ void bar_sync(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
-__device__ __forceinline__ void bar_arrive(int id) { asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory"); }
+// ---- barriers between the two warps of a group (mbarriers in shared memory) ----
+__device__ __forceinline__ unsigned sm_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void mb_init(unsigned b, int warps) {
+  asm volatile("mbarrier.init.shared.b64 [%0], %1;" ::"r"(b), "r"(warps) : "memory");
+}
+// this warp's arrival: what its lanes did before is visible to whoever waits for the phase
+__device__ __forceinline__ void mb_arrive(unsigned b) {
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) asm volatile("mbarrier.arrive.shared.b64 _, [%0];" ::"r"(b) : "memory");
+  __syncwarp();
+}
+// waits for the end of a phase of this parity; false when it has not come after about a second
+__device__ __forceinline__ bool mb_wait(unsigned b, int parity) {
+  unsigned done = 0;
+  for (int i = 0; !done && i < (1 << 20); ++i)
+    asm volatile("{\n .reg .pred q;\n mbarrier.try_wait.parity.shared.b64 q, [%1], %2;\n selp.u32 %0, 1, 0, q;\n}"
+                 : "=r"(done)
+                 : "r"(b), "r"(parity & 1)
+                 : "memory");
+  __syncwarp();
+  return done != 0;
+}
 
 __device__ __forceinline__ void mag_or(unsigned& m, i64 x) {
   const int h = (int)(x >> 32);
@@ -254,6 +274,7 @@ struct FxShared {
   fxc* G;                       // spectrum
   int2 *exA, *exG, *ex1, *ex2;  // lines [k2][k1], slab rows [j][k1], the group's rows and columns
   int *exP, *etA, *etG, *flag;
+  unsigned bar;                 // the group's barriers: read, written, both (8 bytes each)
   double2* T;                   // the warp's line staging (in the slab buffers)
   int warp, lane, grp, wb, ln, sub;
   __device__ __forceinline__ FxShared(unsigned char* smem, fxc* Gglobal) {
@@ -276,6 +297,7 @@ struct FxShared {
     etA = q + C::NG * 64;
     etG = etA + N;
     flag = etG + N;
+    bar = sm_addr(flag + 4) + grp * 24;
     T = reinterpret_cast<double2*>(smem + (size_t)warp * (C::v_bytes / C::NW / 16 * 16));
   }
 };
@@ -283,20 +305,25 @@ struct FxShared {
 // The transforms of a stage, in the order of their data: Phase B per group of slabs (rows forward,
 // the first and the second half of the columns forward and back, rows back), Phase CA per group
 // of lines (back, forward).
+enum FxBar { kRead = 0, kWritten = 8, kBoth = 16 };
 enum FxStep { kRowF, kColF0, kColB0, kColF1, kColB1, kRowB, kLineB, kLineF };
 
+// The halves of a transform are exchanged through the slab buffer three times per group of slabs
+// (columns twice, rows): the odd half signals that it has read its input (barrier kRead), the even
+// half then puts its result there and signals that (kWritten), the odd half adds its own.  Each
+// barrier's phases are told apart by their parity: a phase's one arrival follows its partner's wait
+// for the phase before.  `turn` counts the exchanges.
 // One phase of stage st (st = -1: only the forward lines of the input) on x point xp.  All steps go
 // through one copy of the transform and of its twist: a copy per step would not fit the
 // instruction cache, and two of them already cost 400 bytes of spilled registers.
 template <int N, bool X2>
-__device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, bool lines) {
+__device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, bool lines, int& turn) {
   using C = FxCfg<N>;
   constexpr int L = C::L, SPW = C::SPW, NG = C::NG, NW = C::NW, VR = C::VR, N2 = N * N, N3 = N * N * N;
   constexpr bool GSM = C::GSM;
   extern __shared__ __align__(16) unsigned char smem[];
   const FxShared<N> S(smem, p.G);
   const uint64_t pol = l2_keep_policy(), spol = l2_stream_policy();
-  const int bFull = 1 + 3 * S.grp, bR = 2 + 3 * S.grp, bW = 3 + 3 * S.grp;
   const bool last = st == p.nst - 1, bad = *S.flag != 0, hb = p.base != nullptr;
   double cs = p.coef[0];   // static indexing keeps the parameter block out of local memory
 #pragma unroll
@@ -320,6 +347,7 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
     auto off = [&](int t) { return (size_t)xp * N3 + ((size_t)(t % N) * N + item * SPW + t / N) * N; };
     fxc x[N];
     int E = 0, em = 1;
+    bool ok = true;
 #pragma unroll 1
     for (int step = first; step <= final; ++step) {
       const bool odd = !lines && (step < 3) == (S.wb == 1);   // this warp's half of the padded transform
@@ -345,7 +373,7 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
           const int s = __shfl_sync(0xffffffffu, sh, (S.lane & ~(N - 1)) + n);
           x[n] = {v.re >> s, v.im >> s};
         }
-        if (odd) bar_arrive(bR);   // the columns' entries are read: their place may be written
+        if (odd) mb_arrive(S.bar + kRead);   // the columns' entries are read: their place may be written
       } else if (step == kRowB) {
         const int2 e0 = S.ex2[S.sub * L + S.ln], e1 = S.ex2[S.sub * L + N + S.ln];
         E = align_exp(seg_max<N>(max(e0.x, e1.x)), seg_max<N>(max(e0.y, e1.y)), kFxBits - 1);
@@ -357,7 +385,7 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
           const int s = __shfl_sync(0xffffffffu, sh, (S.lane & ~(N - 1)) + fx_freq<N>(n));
           x[n] = {v.re >> s, v.im >> s};
         }
-        if (odd) bar_arrive(bR);
+        if (odd) mb_arrive(S.bar + kRead);
       } else if (step == kLineB) {
         if (hb) stage_lines<N, X2>(p.base, p.base2, p.cbase2, off, S.T);
         const fxc* g = S.G + (size_t)(item * SPW + S.sub) * N + S.ln;
@@ -399,7 +427,8 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
           row[fx_freq<N>(n)] = x[n];
         }
         S.ex1[(S.sub * 2 + (odd ? 1 : 0)) * N + S.ln] = make_int2(E, E + mag_bits(m));
-        bar_sync(bFull);
+        mb_arrive(S.bar + kBoth);
+        ok &= mb_wait(S.bar + kBoth, 0);
       } else if (step == kColF0 || step == kColF1) {
         const int64_t j = s0 + sc;
         const i64* sg = p.sig + xp * p.sig_xs + ((j * L + (odd ? N : 0)) * L + c);
@@ -420,13 +449,13 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
       } else if (step == kColB0 || step == kColB1) {
         fxc* col = S.V + (size_t)sc * N * VR + c;
         if (!odd) {
-          bar_sync(bR);
+          ok &= mb_wait(S.bar + kRead, turn);
 #pragma unroll
           for (int n = 0; n < N; ++n) col[n * VR] = x[n];
           S.exP[cc] = E;
-          bar_arrive(bW);
+          mb_arrive(S.bar + kWritten);
         } else {
-          bar_sync(bW);
+          ok &= mb_wait(S.bar + kWritten, turn);
           const int ep = S.exP[cc], et = max(ep, E) + 1;
           const int s0_ = shift_of(et, ep), s1_ = shift_of(et, E);
           unsigned m = 0;
@@ -440,16 +469,20 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
           }
           S.ex2[cc] = make_int2(et, et + mag_bits(m));
         }
-        if (step == kColB1) bar_sync(bFull);
+        ++turn;
+        if (step == kColB1) {
+          mb_arrive(S.bar + kBoth);
+          ok &= mb_wait(S.bar + kBoth, 1);
+        }
       } else if (step == kRowB) {
         fxc* row = S.V + (S.sub * N + S.ln) * VR;
         if (!odd) {
 #pragma unroll
           for (int n = 0; n < N; ++n) row[n] = x[n];
-          bar_arrive(bW);
-          bar_sync(bR);
+          mb_arrive(S.bar + kWritten);
+          ok &= mb_wait(S.bar + kRead, turn);
         } else {
-          bar_sync(bW);
+          ok &= mb_wait(S.bar + kWritten, turn);
           fxc* g = S.G + (size_t)(s0 + S.sub) * N2 + S.ln;
           unsigned m = 0;
 #pragma unroll
@@ -462,6 +495,7 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
           }
           S.exG[(s0 + S.sub) * N + S.ln] = make_int2(E, E + mag_bits(m));
         }
+        ++turn;
       } else if (step == kLineB) {
         // c 2^E as one factor where 2^E is well inside the normal numbers, else in two
         const int em_ = max(-800, min(800, E));
@@ -491,6 +525,7 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
         S.exA[(item * SPW + S.sub) * N + S.ln] = make_int2(E, E + mag_bits(m));
       }
     }
+    if (!ok) *S.flag = 1;   // an exchange never came: no result rather than a wrong one
   }
 }
 
@@ -498,6 +533,13 @@ template <int N, bool X2>
 __global__ void __launch_bounds__(FxCfg<N>::NT, 1) k_theta_fx(const FxParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
   const FxShared<N> S(smem, p.G);
+  if (threadIdx.x < FxCfg<N>::NG) {
+    const unsigned b = sm_addr(S.flag + 4) + threadIdx.x * 24;
+    mb_init(b + kRead, 1);
+    mb_init(b + kWritten, 1);
+    mb_init(b + kBoth, 2);
+  }
+  int turn = 0;
   for (int64_t xp = blockIdx.x; xp < p.nxp; xp += gridDim.x) {
     if (threadIdx.x == 0) *S.flag = 0;
     __syncthreads();
@@ -505,7 +547,7 @@ __global__ void __launch_bounds__(FxCfg<N>::NT, 1) k_theta_fx(const FxParams p) 
     for (int ph = 1; ph < 2 * p.nst + 2; ++ph) {   // lines of the input, then slabs and lines per stage
       const int st = ph / 2 - 1;
       const bool lines = ph & 1;
-      fx_phase<N, X2>(p, xp, st, lines);
+      fx_phase<N, X2>(p, xp, st, lines, turn);
       __syncthreads();
       if (st < p.nst - 1 || !lines) {
         align_all<N>(lines ? S.exA : S.exG, lines ? S.etA : S.etG, kFxBits);
