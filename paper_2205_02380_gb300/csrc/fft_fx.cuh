@@ -74,8 +74,21 @@ __device__ __forceinline__ void xfor(F&& f) {
 }
 
 // ---- products ----
-// x w for a constant w = C / 2^64 < 1/2, rounded down to within two units.  The constant's low
-// word is taken as signed, so both cross terms are single high products.
+// a b in 64 bits.  Written as its two halves: the compiler issues one wide product for them, and
+// four instructions for the C expression of the same product.
+__device__ __forceinline__ i64 fx_wide(int a, int b) {
+  int hi;
+  unsigned lo;
+  i64 r;
+  asm("mul.hi.s32 %0, %1, %2;" : "=r"(hi) : "r"(a), "r"(b));
+  asm("mul.lo.s32 %0, %1, %2;" : "=r"(lo) : "r"(a), "r"(b));
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
+  return r;
+}
+// x w for a constant w = C / 2^64 < 1/2, rounded down to within two units; |x| < 2^62.7.  The
+// constant's low word is taken as signed, so both cross terms are single high products.  Their
+// sum fits one word for w < 1/3 (the first is below 2^32 / 3, the second below 2^29.7 in
+// magnitude).
 template <u64 C>
 __device__ __forceinline__ i64 fx_mulc(i64 x) {
   static_assert(C < (1ULL << 63) - (1ULL << 32), "constants below one half");
@@ -83,8 +96,12 @@ __device__ __forceinline__ i64 fx_mulc(i64 x) {
   constexpr unsigned wh = (unsigned)((C >> 32) + (((unsigned)C) >> 31));
   const int xh = (int)(x >> 32);
   const unsigned xl = (unsigned)x;
-  const i64 r = (i64)(int)wh * (i64)xh + (i64)(u64)__umulhi(wh, xl);
-  return r + (i64)__mulhi(wl, xh);
+  const int b = __mulhi(wl, xh);
+  if constexpr (wh < 0x55555555u) {
+    return fx_wide((int)wh, xh) + (i64)(int)(__umulhi(wh, xl) + (unsigned)b);
+  } else {
+    return fx_wide((int)wh, xh) + (i64)(u64)__umulhi(wh, xl) + (i64)b;
+  }
 }
 // a +- x w, 0 <= w <= 1 given as C / 2^64
 template <bool NEG, u64 C>

@@ -9,12 +9,12 @@
 // exponent.
 //
 // Bound.  The FP64 pipe (1.7 FMAs per clock and SM, measured) held the FP64 form of this kernel at
-// 94 % of what its 6.7e6 FP64 instructions per x point and stage allow at N_k = 32; the integer
-// form needs about 3e7 operations of the 60-per-clock integer pipe (a 32-point transform takes 20
-// clocks per thread and SM against 231) and runs at about 60 % of that pipe, waiting for the
-// L2-resident spectrum, the symbol and the slab buffers with two warps per scheduler (64-bit
-// vectors of 32 complex values leave no registers for more).  P(dt): 224.3 -> 43.5 ms at
-// 16^3 x 32^3, 77.7 -> 13.4 ms at 24^3 x 16^3.
+// 94 % of what its 6.7e6 FP64 instructions per x point and stage allow at N_k = 32.  The integer
+// form issues in 40 % of the cycles (ncu at 640 x points, N_k = 32: integer pipe 40 %, multiplier
+// 35 %); two warps per scheduler, all that 64-bit vectors of 32 complex values leave registers
+// for, wait for their own results (1.06 warps per issue), for the L2-resident spectrum and the
+// symbol (0.60), and for instructions (0.56: 181 KB of code).  P(dt): 224.3 -> 37.3 ms at
+// 16^3 x 32^3, 77.7 -> 12.3 ms at 24^3 x 16^3.
 //
 // Errors.  A vector enters a transform with 57 bits below its largest entry and leaves it with an
 // error of about 3 units of the last of them, so each of the eight transforms of a stage adds
@@ -32,7 +32,7 @@
 //   Phase CA  lines along k3: inverse, Theta, Horner update, and for all but the last stage the
 //             forward transform of the new iterate.
 // Inverse transforms run the forward code on (im, re), and all steps of both phases go through one
-// copy of it (two copies: 53.8 ms at 16^3 x 32^3, mostly spilled registers).
+// copy of it: the instruction cache and the registers do not hold two.
 // Layouts: spectrum G[j][k2][k1] (k1 fastest: a warp's rows and its lines along k3 are both
 // consecutive), in shared memory for N <= 16 and in an L2-resident scratch otherwise; slab buffer
 // V[row][2N + 1] per slab; exponents beside them, one per vector.
@@ -59,7 +59,6 @@ struct FxParams {
   const int16_t* sigx; // [nxp][N][2][2N] its exponents
   int64_t sigx_xs;
   int nst;             // stages, 1..4
-  int real;            // 1: real spectrum of an even kernel (the plain TKM convolution)
   double coef[4];      // c_s per stage
   fxc* G;              // per-CTA spectrum scratch when it is not in shared memory
 };
@@ -158,8 +157,10 @@ __device__ __forceinline__ void prefetch_l2(const void* src, unsigned bytes) {
 __device__ __forceinline__ i64 fx_mulsym(i64 x, i64 y) {
   const int xh = (int)(x >> 32), yh = (int)(y >> 32), yl = (int)y;
   const unsigned xl = (unsigned)x;
-  const int a = (int)(__umulhi((unsigned)yh, xl) - (xl & (unsigned)(yh >> 31)));
-  return (i64)xh * (i64)yh + (i64)a + (i64)__mulhi(yl, xh);
+  // the cross terms: signed high times unsigned low word (below 2^30 in magnitude: |yh| <= 2^30),
+  // and signed times signed (below 2^29.7)
+  const int t = (int)(__umulhi((unsigned)yh, xl) - (xl & (unsigned)(yh >> 31)) + (unsigned)__mulhi(yl, xh));
+  return fx_wide(xh, yh) + (i64)t;
 }
 
 // The lines of one warp (N doubles each, line of lane t at src + off(t)) into a staging buffer,
@@ -181,6 +182,11 @@ __device__ __forceinline__ void stage_lines(const double* src, const double* src
     T[t * TR + e] = v;
   }
   __syncwarp();
+}
+template <int N>
+__device__ __forceinline__ void clear_line(double* row) {
+#pragma unroll
+  for (int n = 0; n < N; ++n) row[n] = 0.0;
 }
 template <int N, class Off>
 __device__ __forceinline__ void unstage_lines(double* dst, Off&& off, const double2* T) {
@@ -230,18 +236,16 @@ __device__ __forceinline__ int quantise_line(const double* row, int em, fxc (&x)
 
 // sin phi Re z + cos phi Im z (the real part of -i e^{i phi} ... with the symbol's factor i taken
 // out), or cos phi Re z - sin phi Im z for a real spectrum; phi = pi n / (2N)
-template <int N, int n>
-__device__ __forceinline__ i64 untwist(i64 re, i64 im, bool real) {
-  const i64 a = real ? re : im;          // times cos
-  const i64 b = real ? -im : re;         // times sin
+template <int N, int n, bool REAL>
+__device__ __forceinline__ i64 untwist(i64 re, i64 im) {
   if constexpr (n == 0) {
-    return a;
+    return REAL ? re : im;
   } else {
     constexpr bool up = 8 * n > 4 * N;
     constexpr int k = up ? N - n : n;
     constexpr u64 c = up ? FxK<k, 4 * N>::sin : FxK<k, 4 * N>::cos;
     constexpr u64 s = up ? FxK<k, 4 * N>::cos : FxK<k, 4 * N>::sin;
-    return fx_mul<c>(a) + fx_mul<s>(b);
+    return REAL ? fx_mul<c>(re) - fx_mul<s>(im) : fx_mul<c>(im) + fx_mul<s>(re);
   }
 }
 
@@ -314,9 +318,11 @@ enum FxStep { kRowF, kColF0, kColB0, kColF1, kColB1, kRowB, kLineB, kLineF };
 // barrier's phases are told apart by their parity: a phase's one arrival follows its partner's wait
 // for the phase before.  `turn` counts the exchanges.
 // One phase of stage st (st = -1: only the forward lines of the input) on x point xp.  All steps go
-// through one copy of the transform and of its twist: a copy per step would not fit the
-// instruction cache, and two of them already cost 400 bytes of spilled registers.
-template <int N, bool X2>
+// through one copy of the transform's middle part: a copy per step would not fit the
+// instruction cache, and two of them already cost 400 bytes of spilled registers (53.8 against
+// 49.3 ms at 16^3 x 32^3).
+// REAL: real spectrum of an even kernel (the plain TKM convolution).
+template <int N, bool X2, bool REAL>
 __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, bool lines, int& turn) {
   using C = FxCfg<N>;
   constexpr int L = C::L, SPW = C::SPW, NG = C::NG, NW = C::NW, VR = C::VR, N2 = N * N, N3 = N * N * N;
@@ -324,12 +330,13 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
   extern __shared__ __align__(16) unsigned char smem[];
   const FxShared<N> S(smem, p.G);
   const uint64_t pol = l2_keep_policy(), spol = l2_stream_policy();
-  const bool last = st == p.nst - 1, bad = *S.flag != 0, hb = p.base != nullptr;
+  const bool last = st == p.nst - 1, bad = *S.flag != 0;
   double cs = p.coef[0];   // static indexing keeps the parameter block out of local memory
 #pragma unroll
   for (int q = 1; q < 4; ++q)
     if (q == st) cs = p.coef[q];
-  if (!p.real) cs = -cs;
+  if (!REAL) cs = -cs;
+  if (bad) cs = __longlong_as_double(0x7ff8000000000000LL);
   double* row = reinterpret_cast<double*>(S.T + S.lane * C::TROW);   // this lane's line
   const int first = lines ? (st < 0 ? kLineF : kLineB) : kRowF;
   const int final = lines ? (last ? kLineB : kLineF) : kRowB;
@@ -387,7 +394,8 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
         }
         if (odd) mb_arrive(S.bar + kRead);
       } else if (step == kLineB) {
-        if (hb) stage_lines<N, X2>(p.base, p.base2, p.cbase2, off, S.T);
+        if (p.base) stage_lines<N, X2>(p.base, p.base2, p.cbase2, off, S.T);
+        else clear_line<N>(row);
         const fxc* g = S.G + (size_t)(item * SPW + S.sub) * N + S.ln;
 #pragma unroll
         for (int n = 0; n < N; ++n) {
@@ -500,14 +508,12 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
         // c 2^E as one factor where 2^E is well inside the normal numbers, else in two
         const int em_ = max(-800, min(800, E));
         const double c2 = cs * pow2_mid(em_), rest = pow2_mid(max(-900, min(900, E - em_)));
-        const bool real = p.real != 0;
         em = 1;
         xfor<0, N>([&](auto I) {
           constexpr int n = decltype(I)::value;
-          double th = (double)untwist<N, n>(x[n].im, x[n].re, real);
+          double th = (double)untwist<N, n, REAL>(x[n].im, x[n].re);
           if (em_ != E) th *= rest;
-          double v = fma(c2, th, hb ? row[n] : 0.0);
-          if (bad) v = __longlong_as_double(0x7ff8000000000000LL);
+          const double v = fma(c2, th, row[n]);
           em = max(em, (__double2hiint(v) >> 20) & 0x7ff);
           row[n] = v;
           asm volatile("" ::: "memory");   // one entry after the other: there are no registers to spare
@@ -529,7 +535,7 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
   }
 }
 
-template <int N, bool X2>
+template <int N, bool X2, bool REAL>
 __global__ void __launch_bounds__(FxCfg<N>::NT, 1) k_theta_fx(const FxParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
   const FxShared<N> S(smem, p.G);
@@ -547,7 +553,7 @@ __global__ void __launch_bounds__(FxCfg<N>::NT, 1) k_theta_fx(const FxParams p) 
     for (int ph = 1; ph < 2 * p.nst + 2; ++ph) {   // lines of the input, then slabs and lines per stage
       const int st = ph / 2 - 1;
       const bool lines = ph & 1;
-      fx_phase<N, X2>(p, xp, st, lines, turn);
+      fx_phase<N, X2, REAL>(p, xp, st, lines, turn);
       __syncthreads();
       if (st < p.nst - 1 || !lines) {
         align_all<N>(lines ? S.exA : S.exG, lines ? S.etA : S.etG, kFxBits);
@@ -585,10 +591,11 @@ __global__ void k_fx_symbol(i64* __restrict__ sig, int16_t* __restrict__ ex, int
 template <int N>
 void plan_fx_n(int64_t nxp, int num_sms, ThetaPlan* pl) {
   using C = FxCfg<N>;
-  cudaFuncSetAttribute(k_theta_fx<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_bytes);
-  cudaFuncSetAttribute(k_theta_fx<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_bytes);
+  cudaFuncSetAttribute(k_theta_fx<N, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_bytes);
+  cudaFuncSetAttribute(k_theta_fx<N, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_bytes);
+  cudaFuncSetAttribute(k_theta_fx<N, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_bytes);
   int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_theta_fx<N, false>, C::NT, C::smem_bytes) != cudaSuccess || nb < 1)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_theta_fx<N, false, false>, C::NT, C::smem_bytes) != cudaSuccess || nb < 1)
     nb = 1;
   pl->cluster = 0;
   pl->blocks = (int)std::min<int64_t>(nxp, (int64_t)nb * num_sms);
@@ -614,11 +621,16 @@ cudaError_t launch_fx_n(const Handle& H, const void* in, const void* base, void*
   p.sig_xs = x.sig ? 0 : per;
   p.sigx_xs = x.sig ? 0 : (int64_t)N * 2 * C::L;
   p.nst = nst;
-  p.real = x.real_symbol ? 1 : 0;
   for (int q = 0; q < 4; ++q) p.coef[q] = q < nst ? coef[q] : 0.0;
   p.G = static_cast<fxc*>(H.d_scratch);
-  if (x.in2 || x.base2) k_theta_fx<N, true><<<H.theta.blocks, C::NT, C::smem_bytes, s>>>(p);
-  else k_theta_fx<N, false><<<H.theta.blocks, C::NT, C::smem_bytes, s>>>(p);
+  if (x.real_symbol) {
+    if (x.in2 || x.base2) return cudaErrorInvalidValue;
+    k_theta_fx<N, false, true><<<H.theta.blocks, C::NT, C::smem_bytes, s>>>(p);
+  } else if (x.in2 || x.base2) {
+    k_theta_fx<N, true, false><<<H.theta.blocks, C::NT, C::smem_bytes, s>>>(p);
+  } else {
+    k_theta_fx<N, false, false><<<H.theta.blocks, C::NT, C::smem_bytes, s>>>(p);
+  }
   return cudaGetLastError();
 }
 
