@@ -21,10 +21,14 @@
 // about 48 significant bits), i.e. at FP64-class precision without the FP64 pipe, which on GB300
 // delivers 1/64 of the FP32 rate and otherwise bounds this pass.  Everything else is FP32.
 //
-// Two kernels: k_advect_reg keeps the line in registers (line length a compile-time constant
-// from {16, 24, 32, 48, 64} and integer shift in [-2, 1], the usual case since |alpha| < 1);
-// k_advect_smem is the general fallback with the line in shared memory (column layout, element
-// e of thread t at e*B + t, conflict-free).
+// Two kernels: k_advect_reg keeps the line in registers (integer shift in [-2, 1], the usual case
+// since |alpha| < 1; line length a compile-time constant from {16, 24, 32, 48, 64}, and in FP32
+// any length up to 64, in classes of four); k_advect_smem is the general fallback with the line
+// in shared memory (column layout, element e of thread t at e*B + t, conflict-free).
+// FP32 lengths between the constants ran in shared memory before, bound by its round trips: A(tau)
+// on 20^3, 36^2 x 16 and 60^2 x 16 x 32^3 at 2.37, 3.11 and 2.79 TB/s per pass, now 5.63, 5.35 and
+// 5.03 (32 points: 6.11).  FP64 is bound by the FP64 pipe, where the padded slots cost more than
+// shared memory does: ragged registers 661, 807 and 868 GB/s, shared memory 985, 907 and 893.
 #include <cstring>
 
 #include "internal.hpp"
@@ -213,6 +217,55 @@ __device__ __forceinline__ void solve_line(const AdvParams<T>& p, const AdvTabs<
   v[N + 2] = (T)cl.gr(v[N], h2val(p));
 }
 
+// The same for a line of n points, NX - kRag < n <= NX: everything keeps its compile-time slot,
+// what depends on the line's end is selected among the last kRag slots.  The right stencil is
+// stored by node (tb.c[..][i] multiplies phi_i); the factors are zero beyond N, so the slots there
+// become zero and take no part.  The leading taps of the right stencil may start anywhere in that
+// window, so kClosHead + kRag - 1 of them are accumulated error-free.  Classes of four: with
+// classes of eight 25 points ran at 4.04 TB/s per pass (5.53), 17 points at 4.00 (5.04).
+constexpr int kRag = 4;
+__device__ __forceinline__ void closure_left(Closure<float>& cl, const AdvTabs<float>& tb, int j, float phi) {
+  if (j < kClosHead) df_acc(cl.L, phi, tb.c[0][j], tb.c[1][j]);
+  else cl.L.lo = fmaf(phi, tb.c[0][j], cl.L.lo);
+}
+template <int NX>
+__device__ __forceinline__ void closure_right(Closure<float>& cl, const AdvTabs<float>& tb, int i, float phi) {
+  if (i >= NX - kRag + 1 - kClosHead) df_acc(cl.R, phi, tb.c[2][i], tb.c[3][i]);
+  else cl.R.lo = fmaf(phi, tb.c[2][i], cl.R.lo);
+}
+template <typename T, int NX, int JC>
+__device__ __forceinline__ void solve_ragged(const AdvParams<T>& p, const AdvTabs<T>& tb, T (&v)[NX + 2]) {
+  const int N = p.n - 1;
+  constexpr int W0 = NX > kRag ? NX - kRag : 0;   // first slot the line may end at
+  Closure<T> cl;
+#pragma unroll
+  for (int j = 0; j < JC; ++j) closure_left(cl, tb, j, v[j + 1]);
+#pragma unroll
+  for (int i = NX - 1; i >= 0; --i)
+    if (i > W0 - JC) closure_right<NX>(cl, tb, i, v[i + 1]);
+  T dp = (T)cl.d0(v[1], hval(p)) * tb.lu[1][0];
+  v[1] = dp;
+#pragma unroll
+  for (int i = 1; i < NX; ++i) {
+    T r = (T)6 * v[i + 1];
+    if (i >= W0 && i == N) r = (T)cl.dN(v[i + 1], hval(p));
+    dp = (r - dp) * tb.lu[1][i];
+    v[i + 1] = dp;
+  }
+#pragma unroll
+  for (int i = NX - 2; i >= 0; --i) v[i + 1] = v[i + 1] - tb.lu[0][i] * v[i + 2];
+  v[0] = (T)cl.gl(v[2], h2val(p));
+#pragma unroll
+  for (int i = W0 > 1 ? W0 : 1; i < NX; ++i)
+    if (i == N) v[i + 2] = (T)cl.gr(v[i], h2val(p));
+}
+template <typename T, int NX, int JC, bool RAG>
+__device__ __forceinline__ void solve_any(const AdvParams<T>& p, const AdvTabs<T>& tb, T (&v)[NX + 2]) {
+  static_assert(!RAG || sizeof(T) == 4, "ragged lengths: FP32");
+  if constexpr (RAG) solve_ragged<T, NX, JC>(p, tb, v);
+  else solve_line<T, NX, JC>(p, tb, v);
+}
+
 // the 4-tap evaluation of two lines with the same integer shift S (weights wa, wb), written
 // together by st(j, out_a, out_b)
 template <typename T, int NX, int S, class St>
@@ -242,11 +295,11 @@ __device__ __forceinline__ void eval_line2(const T (&va)[NX + 2], const T (&vb)[
   }
 }
 
-// solve_line, then the 4-tap evaluation at the feet of line k index kd, written by st
-template <typename T, int NX, int JC, class St>
+// the solve, then the 4-tap evaluation at the feet of line k index kd, written by st
+template <typename T, int NX, int JC, bool RAG, class St>
 __device__ __forceinline__ void solve_eval_line(const AdvParams<T>& p, const AdvTabs<T>& tb,
                                                 T (&v)[NX + 2], int kd, St&& st) {
-  solve_line<T, NX, JC>(p, tb, v);
+  solve_any<T, NX, JC, RAG>(p, tb, v);
   const int sh = __ldg(p.ns + kd);
   const T w0 = __ldg(p.w + 4 * kd + 0), w1 = __ldg(p.w + 4 * kd + 1);
   const T w2 = __ldg(p.w + 4 * kd + 2), w3 = __ldg(p.w + 4 * kd + 3);
@@ -262,7 +315,7 @@ __device__ __forceinline__ void solve_eval_line(const AdvParams<T>& p, const Adv
 // x indices) per thread, loaded with 8-byte accesses so each thread keeps twice the bytes in
 // flight, and stored with 8-byte accesses when both lines have the same integer shift (always
 // for the x1 and x2 passes, whose shift depends on k1 or k2 only).
-template <typename T, int NX, int JC>
+template <typename T, int NX, int JC, bool RAG>
 __global__ void __launch_bounds__(kAdvectThreads) k_advect_reg(AdvParams<T> p, const AdvTabs<T> tb) {
   constexpr int LPT = sizeof(T) == 4 ? 2 : 1;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -270,37 +323,45 @@ __global__ void __launch_bounds__(kAdvectThreads) k_advect_reg(AdvParams<T> p, c
   T* src;
   int kd;
   line_setup(p, t * LPT, src, kd);
+  auto in_line = [&](int j) { return !RAG || j < NX - kRag || j < p.n; };   // n > NX - kRag
   if constexpr (LPT == 1) {
     T v[NX + 2];   // slot nu + 1 holds eta_nu (phi_j before the solve)
 #pragma unroll
     for (int j = 0; j < NX; ++j) v[j + 1] = src[(int64_t)j * p.s_d];
-    solve_eval_line<T, NX, JC>(p, tb, v, kd, [&](int j, T o) { src[(int64_t)j * p.s_d] = o; });
+    solve_eval_line<T, NX, JC, RAG>(p, tb, v, kd, [&](int j, T o) { src[(int64_t)j * p.s_d] = o; });
   } else {
     T v0[NX + 2], v1[NX + 2];
 #pragma unroll
     for (int j = 0; j < NX; ++j) {
-      const float2 q = *reinterpret_cast<const float2*>(src + (int64_t)j * p.s_d);
+      const float2 q = in_line(j) ? *reinterpret_cast<const float2*>(src + (int64_t)j * p.s_d) : make_float2(0.f, 0.f);
       v0[j + 1] = q.x;
       v1[j + 1] = q.y;
     }
+    if constexpr (RAG) v0[0] = v0[NX + 1] = v1[0] = v1[NX + 1] = (T)0;
     int kd1;
     T* src1;
     line_setup(p, t * LPT + 1, src1, kd1);
     const int sh0 = __ldg(p.ns + kd), sh1 = __ldg(p.ns + kd1);
     if (sh0 != sh1) {   // rare: the two k straddle an integer shift
-      solve_eval_line<T, NX, JC>(p, tb, v0, kd, [&](int j, T o) { src[(int64_t)j * p.s_d] = o; });
-      solve_eval_line<T, NX, JC>(p, tb, v1, kd1, [&](int j, T o) { src1[(int64_t)j * p.s_d] = o; });
+      solve_eval_line<T, NX, JC, RAG>(p, tb, v0, kd, [&](int j, T o) {
+        if (in_line(j)) src[(int64_t)j * p.s_d] = o;
+      });
+      solve_eval_line<T, NX, JC, RAG>(p, tb, v1, kd1, [&](int j, T o) {
+        if (in_line(j)) src1[(int64_t)j * p.s_d] = o;
+      });
       return;
     }
-    solve_line<T, NX, JC>(p, tb, v0);
-    solve_line<T, NX, JC>(p, tb, v1);
+    solve_any<T, NX, JC, RAG>(p, tb, v0);
+    solve_any<T, NX, JC, RAG>(p, tb, v1);
     T wa[4], wb[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       wa[c] = __ldg(p.w + 4 * kd + c);
       wb[c] = __ldg(p.w + 4 * kd1 + c);
     }
-    auto st = [&](int j, T a, T b) { *reinterpret_cast<float2*>(src + (int64_t)j * p.s_d) = make_float2(a, b); };
+    auto st = [&](int j, T a, T b) {
+      if (in_line(j)) *reinterpret_cast<float2*>(src + (int64_t)j * p.s_d) = make_float2(a, b);
+    };
     switch (sh0) {
       case -2: eval_line2<T, NX, -2>(v0, v1, wa, wb, st); break;
       case -1: eval_line2<T, NX, -1>(v0, v1, wa, wb, st); break;
@@ -491,23 +552,25 @@ AdvParams<T> make_params(const Handle& H, void* f, int dim) {
   return p;
 }
 
-// closure stencils and Thomas factors of dimension dim for the register kernels
+// closure stencils and Thomas factors of dimension dim for the register kernels (ragged: the
+// right stencil by node instead of by distance from the end)
 template <typename T>
-AdvTabs<T> make_tabs(const Handle& H, int dim) {
+AdvTabs<T> make_tabs(const Handle& H, int dim, bool ragged) {
   const int n = H.g.nx[dim];
   AdvTabs<T> tb;
   std::memset(&tb, 0, sizeof(tb));
   const std::vector<double>& hc = H.h_clos[dim];
   const std::vector<double>& hl = H.h_lu[dim];
   for (int j = 0; j < n; ++j) {
+    const int jr = ragged ? n - 1 - j : j;
     if constexpr (sizeof(T) == 4) {   // unevaluated float pairs hi + lo of the FP64 stencils
       tb.c[0][j] = (float)hc[j];
       tb.c[1][j] = (float)(hc[j] - (double)tb.c[0][j]);
-      tb.c[2][j] = (float)hc[n + j];
-      tb.c[3][j] = (float)(hc[n + j] - (double)tb.c[2][j]);
+      tb.c[2][j] = (float)hc[n + jr];
+      tb.c[3][j] = (float)(hc[n + jr] - (double)tb.c[2][j]);
     } else {
       tb.c[0][j] = hc[j];
-      tb.c[1][j] = hc[n + j];
+      tb.c[1][j] = hc[n + jr];
     }
     tb.lu[0][j] = (T)hl[j];
     tb.lu[1][j] = (T)hl[n + j];
@@ -515,10 +578,32 @@ AdvTabs<T> make_tabs(const Handle& H, int dim) {
   return tb;
 }
 
-// the register kernels apply: integer shifts in [-2, 1] and a compiled line length
-bool reg_applies(const Handle& H, int dim) {
+// The register kernels apply: integer shifts in [-2, 1], up to kRegMaxNx points and (in FP32, for
+// the 8-byte accesses) an even address.
+bool reg_applies(const Handle& H, const void* f, int dim) {
   return H.adv.ns_min[dim] >= -2 && H.adv.ns_max[dim] <= 1 && H.opt.patches[dim] <= 1 &&
-         H.g.nx[dim] <= kRegMaxNx;
+         H.g.nx[dim] <= kRegMaxNx && (reinterpret_cast<uintptr_t>(f) & 7) == 0;
+}
+
+// Lines of n points with their length a compile-time constant (the workloads' lengths)
+template <typename T, int NX>
+void launch_exact(const AdvParams<T>& p, const AdvTabs<T>& tb, unsigned blocks, cudaStream_t s) {
+  // closure taps: the launch's J rounded up to a compiled bucket (the stencil is zero beyond J)
+  constexpr int JS = NX > 24 ? 24 : NX;
+  if (p.J <= JS) k_advect_reg<T, NX, JS, false><<<blocks, kAdvectThreads, 0, s>>>(p, tb);
+  else k_advect_reg<T, NX, NX, false><<<blocks, kAdvectThreads, 0, s>>>(p, tb);
+}
+// NX - kRag < n <= NX, J <= 24, FP32
+template <int NX>
+bool launch_ragged(const AdvParams<float>& p, const AdvTabs<float>& tb, unsigned blocks, cudaStream_t s) {
+  if constexpr (NX < 4) {
+    return false;
+  } else {
+    if (p.n <= NX - kRag) return launch_ragged<NX - kRag>(p, tb, blocks, s);
+    constexpr int JS = NX > 24 ? 24 : NX;
+    k_advect_reg<float, NX, JS, true><<<blocks, kAdvectThreads, 0, s>>>(p, tb);
+    return true;
+  }
 }
 
 template <typename T>
@@ -541,28 +626,23 @@ cudaError_t launch_t(const Handle& H, void* f, int dim, cudaStream_t s) {
     k_advect_patches<T><<<(unsigned)((p.n_lines + Bp - 1) / Bp), Bp, elems * Bp * sizeof(T), s>>>(p, q);
     return cudaGetLastError();
   }
-  if (reg_applies(H, dim)) {
+  if (reg_applies(H, f, dim)) {
     const int64_t lpt = sizeof(T) == 4 ? 2 : 1;   // kvol = nk^3 is even
     const unsigned rblocks = (unsigned)((p.n_lines / lpt + B - 1) / B);
-    const AdvTabs<T> tb = make_tabs<T>(H, dim);
-    // closure taps: the launch's J rounded up to a compiled bucket (the stencil is zero beyond J)
-    const bool short_j = p.J <= 24 && p.n > 24;
-#define CHASM_REG(NX)                                                                   \
-  case NX:                                                                              \
-    if (short_j && NX > 24)                                                             \
-      k_advect_reg<T, NX, (NX > 24 ? 24 : NX)><<<rblocks, B, 0, s>>>(p, tb);            \
-    else                                                                                \
-      k_advect_reg<T, NX, NX><<<rblocks, B, 0, s>>>(p, tb);                             \
-    return cudaGetLastError();
-    switch (p.n) {
-      CHASM_REG(16)
-      CHASM_REG(24)
-      CHASM_REG(32)
-      CHASM_REG(48)
-      CHASM_REG(64)
-      default: break;
+    const bool exact = p.n == 16 || p.n == 24 || p.n == 32 || p.n == 48 || p.n == 64;
+    if (exact || (sizeof(T) == 4 && p.J <= 24)) {
+      const AdvTabs<T> tb = make_tabs<T>(H, dim, !exact);
+      switch (p.n) {
+        case 16: launch_exact<T, 16>(p, tb, rblocks, s); break;
+        case 24: launch_exact<T, 24>(p, tb, rblocks, s); break;
+        case 32: launch_exact<T, 32>(p, tb, rblocks, s); break;
+        case 48: launch_exact<T, 48>(p, tb, rblocks, s); break;
+        case 64: launch_exact<T, 64>(p, tb, rblocks, s); break;
+        default:
+          if constexpr (sizeof(T) == 4) launch_ragged<kRegMaxNx>(p, tb, rblocks, s);
+      }
+      return cudaGetLastError();
     }
-#undef CHASM_REG
   }
   const size_t elems = advect_smem_elems(g.nx[dim], 1);
   const int Bs = advect_smem_threads(elems, sizeof(T));
