@@ -396,6 +396,22 @@ int ensure_kshift_rows(Handle* H, double dt) {
   int rc;
   if (H->fp64) {
     rc = upload_real(H, &H->d_krows, rows);
+    // the spectra phi_m in FFT order (re, im), for the transforms of k_kpass_fx.cu
+    std::vector<int64_t> spec((size_t)tot * 2 * N);
+    id = 0;
+    for (int d = 0; d < 3; ++d)
+      for (int i = 0; i < H->g.nx[d]; ++i, ++id) {
+        const double s = dt * H->kappa * (H->g.x_lo[d] + i * H->g.h[d] - H->center[d]) / H->hbar;
+        for (int q = 0; q < N; ++q) {
+          const int mm = q < N / 2 ? q : q - N;
+          const double a = M_PI * mm / H->g.lk * s;
+          spec[((size_t)id * N + q) * 2] = fx_spec_entry(std::cos(a));
+          spec[((size_t)id * N + q) * 2 + 1] = fx_spec_entry(2 * q == N ? 0.0 : std::sin(a));
+        }
+      }
+    if (rc == CHASM_OK) rc = upload(H, &H->d_kspec, spec.data(), spec.size() * sizeof(int64_t));
+    if (rc == CHASM_OK && cudaStreamSynchronize(H->stream) != cudaSuccess)
+      rc = fail(H, CHASM_ECUDA, "k-shift table upload");
   } else {   // the columns of the circulant sum to 1: keep that in FP32 (mass of the k-shift)
     std::vector<float> rf(rows.size());
     for (int r = 0; r < tot; ++r) round_unit_sum(&rows[(size_t)r * N], &rf[(size_t)r * N], N);
@@ -406,6 +422,26 @@ int ensure_kshift_rows(Handle* H, double dt) {
   if (rc) return rc;
   H->krows_dt = dt;
   H->krows_valid = true;
+  return CHASM_OK;
+}
+
+// FP64: the spectral k-derivative of the quadratic potential, its circulant column d_j = -(2/N)
+// sum_{m=1}^{N/2-1} xi_m sin(2 pi m j / N) and its spectrum xi_m / max xi in FFT order (the Nyquist
+// mode dropped).
+int build_kderiv(Handle* H) {
+  const int N = H->g.nk;
+  std::vector<int64_t> t(2 * (size_t)N);
+  for (int j = 0; j < N; ++j) {
+    double acc = 0.0;
+    for (int m = 1; m < N / 2; ++m) acc += (M_PI * m / H->g.lk) * std::sin(2.0 * M_PI * m * j / N);
+    const double d = -2.0 * acc / N;
+    std::memcpy(&t[j], &d, sizeof(d));
+    const int m = j < N / 2 ? j : j - N;
+    t[N + j] = fx_spec_entry(2 * j == N ? 0.0 : (double)m / (N / 2 - 1));
+  }
+  int rc = upload(H, &H->d_kderiv, t.data(), t.size() * sizeof(int64_t));
+  if (rc) return rc;
+  CHASM_CUDA(H, cudaStreamSynchronize(H->stream));
   return CHASM_OK;
 }
 
@@ -504,7 +540,7 @@ void free_all(Handle* H) {
   void* ptrs[] = {H->d_clos[0], H->d_clos[1], H->d_clos[2], H->d_lu[0], H->d_lu[1], H->d_lu[2],
                   H->d_pclos[0], H->d_pclos[1], H->d_pclos[2], H->d_plu[0], H->d_plu[1], H->d_plu[2],
                   H->adv.dev, H->d_T,
-                  H->d_that, H->d_phase, H->d_sig, H->d_tkm, H->d_scratch, H->d_u[0], H->d_u[1], H->d_krows,
+                  H->d_that, H->d_phase, H->d_sig, H->d_tkm, H->d_scratch, H->d_u[0], H->d_u[1], H->d_krows, H->d_kspec, H->d_kderiv,
                   H->d_partials, H->d_result, H->d_vx, H->d_diag, H->d_fhost};
   for (void* p : ptrs)
     if (p) cudaFreeAsync(p, H->stream);
@@ -725,7 +761,7 @@ size_t chasm_workspace_bytes(const chasm_grid* grid, const chasm_potential* pot,
   w += (size_t)nxp * 8 + 3 * (size_t)moments_blocks() * 8 + 64;
   w += diag_bytes(grid->nx, nk);
   w += (size_t)3 * (grid->nx[0] + grid->nx[1] + grid->nx[2]) * (8 + 2 * e);
-  w += (size_t)(grid->nx[0] + grid->nx[1] + grid->nx[2]) * nk * e + 3 * nk * (4 * e + 4);
+  w += (size_t)(grid->nx[0] + grid->nx[1] + grid->nx[2]) * nk * (fp64 ? 24 : 4) + 3 * nk * (4 * e + 4) + 16 * nk;
   return w;
 }
 
@@ -832,6 +868,10 @@ int chasm_create(const chasm_grid* grid, const chasm_box* box, const chasm_poten
           cudaMallocAsync(&H->d_u[1], fbytes, H->stream) != cudaSuccess)
         return bail(fail(H, CHASM_ENOMEM, "device allocation failed (Horner buffers / scratch)"));
     }
+  }
+  if (H->nuclei.empty() && H->kappa != 0.0 && H->fp64) {
+    rc = build_kderiv(H);
+    if (rc) return bail(rc);
   }
   if (o.integrator == CHASM_LPC1 && !H->d_u[0]) {   // LPC1 work copies: Theta f, the predictor
     const bool fused = !H->nuclei.empty() && H->xs;  // the table form forms the predictor in-kernel

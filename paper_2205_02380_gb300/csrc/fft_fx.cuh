@@ -148,6 +148,45 @@ __device__ __forceinline__ fxc fx_rot(fxc z) {
   else return z;
 }
 
+// ---- vectors with a common exponent ----
+// magnitude bits to which the entries of a vector are aligned before a transform (the outputs of
+// two inverse halves are added: one bit less)
+constexpr int kFxBits = 57;
+
+__device__ __forceinline__ void mag_or(unsigned& m, i64 x) {
+  const int h = (int)(x >> 32);
+  m |= (unsigned)(h ^ (h >> 31));
+}
+// number of bits that hold the magnitudes whose high words were or-ed into m
+__device__ __forceinline__ int mag_bits(unsigned m) { return 64 - __clz((int)m); }
+
+// A double as an integer on the scale of a vector whose largest exponent field is em (fields as
+// fx_field gives them, em >= 1): kFxBits bits below the largest entry, magnitudes rounded down.
+// fx_exponent(em) is the exponent of the integers; em = 0x7ff means that an entry is not finite.
+__device__ __forceinline__ int fx_field(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+__device__ __forceinline__ int fx_exponent(int em) { return em - 1023 - (kFxBits - 1); }
+__device__ __forceinline__ i64 fx_from_double(double v, int em) {
+  const int hi = __double2hiint(v), e = fx_field(v);
+  const unsigned mh = (unsigned)(hi & 0xfffff) | (e ? 0x100000u : 0u);
+  u64 m = ((u64)mh << 32 | (unsigned)__double2loint(v)) << (kFxBits - 53);
+  m >>= min(63, em - max(e, 1));
+  const i64 sg = (i64)(hi >> 31);
+  return ((i64)m ^ sg) - sg;
+}
+// 2^e for e in [-900, 900]
+__device__ __forceinline__ double pow2_mid(int e) { return __hiloint2double((e + 1023) << 20, 0); }
+
+// x y / 2^64 for a symbol value y in its stored form: high word, and the low word as a signed
+// number (the high word holds its carry)
+__device__ __forceinline__ i64 fx_mulsym(i64 x, i64 y) {
+  const int xh = (int)(x >> 32), yh = (int)(y >> 32), yl = (int)y;
+  const unsigned xl = (unsigned)x;
+  // the cross terms: signed high times unsigned low word (below 2^30 in magnitude: |yh| <= 2^30),
+  // and signed times signed (below 2^29.7)
+  const int t = (int)(__umulhi((unsigned)yh, xl) - (xl & (unsigned)(yh >> 31)) + (unsigned)__mulhi(yl, xh));
+  return fx_wide(xh, yh) + (i64)t;
+}
+
 // ---- transforms ----
 // DFT_4 in place, natural order: X_j = sum_n x_n e^{-2 pi i jn/4}
 __device__ __forceinline__ void fx_dft4(fxc& a, fxc& b, fxc& c, fxc& d) {

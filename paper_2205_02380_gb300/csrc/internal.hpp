@@ -142,6 +142,13 @@ cudaError_t compute_symbol(int nk, double lk, double* T_dev, void* that_dev, boo
 // misc (k_misc.cu)
 cudaError_t launch_moments(const Handle& H, const void* f, double* partials, double* result_dev,
                            cudaStream_t s);
+// FP64 (k_kpass_fx.cu): one k-dimension of the k-shift (rows, spec: circulant columns and spectra per
+// x_d index) and of Theta of the quadratic potential, out = (add or 0) + coef Theta_d[in];
+// fx_spec_entry: a spectrum value of magnitude at most one in the form those kernels read
+cudaError_t launch_kshift_fx(const Handle& H, void* f, int dim, const void* rows, const void* spec, cudaStream_t s);
+cudaError_t launch_kderiv_fx(const Handle& H, const void* in, const void* add, void* out, int dim, double coef,
+                             cudaStream_t s);
+int64_t fx_spec_entry(double v);
 cudaError_t launch_kshift(const Handle& H, void* f, int dim, const void* rows, cudaStream_t s);
 cudaError_t launch_init_gaussians(const Handle& H, void* f, const chasm_gaussian* g, int n,
                                   cudaStream_t s);
@@ -196,6 +203,8 @@ struct Handle {
   void* d_krows = nullptr;         // circulant rows [3][nx_d][nk] for the current dt
   double krows_dt = 0.0;
   bool krows_valid = false;
+  void* d_kspec = nullptr;         // FP64: the same shifts' spectra (k_kpass_fx.cu)
+  void* d_kderiv = nullptr;        // FP64: the spectral derivative's circulant column and spectrum
   // reductions
   double* d_partials = nullptr;
   double* d_result = nullptr;

@@ -3,11 +3,11 @@
 //   k_kderiv        Theta for V = kappa/2 |x - c|^2 (Eq. 5.1), one k-dimension per launch:
 //                   out = (base or out) + coef kappa (x_d - c_d)/hbar D u along k_d, where D is the
 //                   spectral derivative on the periodic k-grid (i xi_m, xi_m = pi m / L_k, the
-//                   Nyquist mode dropped), applied as its circulant: (D u)_p = sum_j d_j u_{p-j},
-//                   d_j = -(2/N) sum_{m=1}^{N/2-1} xi_m sin(2 pi m j / N).  One thread per k-line
-//                   (two k-adjacent lines in FP32), the N taps in the kernel's parameter block
-//                   (constant-bank operands); the k3 pass (k_kderiv3) stages its contiguous
-//                   lines in shared memory.
+//                   Nyquist mode dropped), in FP32 applied as its circulant: (D u)_p = sum_j d_j u_{p-j},
+//                   d_j = -(2/N) sum_{m=1}^{N/2-1} xi_m sin(2 pi m j / N).  One thread per two
+//                   k-adjacent lines, the N taps in the kernel's parameter block (constant-bank
+//                   operands); the k3 pass (k_kderiv3) stages its contiguous lines in shared
+//                   memory.  FP64 runs k_kpass_fx.cu.
 //   k_lpc1_combine  predictor and corrector base from the advected fields g = f(A_dt) and
 //                   h = Theta[f](A_dt): v = g + dt h (the predictor f~), f = g + dt/2 h.
 #include "internal.hpp"
@@ -29,12 +29,11 @@ struct KDerivParams {
   T d[N];
 };
 
-// FP64: one line per thread.  FP32: two lines per thread, k-adjacent in memory (r even and r + 1,
+// Two lines per thread, k-adjacent in memory (r even and r + 1,
 // the same x point), moved with 8-byte accesses.
 template <typename T, int N>
 __global__ void __launch_bounds__(128) k_kderiv(const KDerivParams<T, N> p) {
-  constexpr int LPT = sizeof(T) == 4 ? 2 : 1;
-  const int64_t line = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * LPT;
+  const int64_t line = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 2;
   if (line >= p.nxp * N * N) return;
   const int64_t xp = line / (N * N);
   const int r = (int)(line % (N * N));
@@ -54,24 +53,7 @@ __global__ void __launch_bounds__(128) k_kderiv(const KDerivParams<T, N> p) {
     id = (int)(xp % p.nx3);
   }
   const T scale = (T)(p.rate_scale * (p.x_lo + id * p.h - p.center)) * p.coef;
-  if constexpr (LPT == 1) {
-    T v[N];
-#pragma unroll
-    for (int l = 0; l < N; ++l) v[l] = p.in[base + l * stride];
-#pragma unroll
-    for (int q = 0; q < N; ++q) {
-      T acc = (T)0;
-#pragma unroll
-      for (int l = 0; l < N; ++l) acc = fma(p.d[(q - l + N) & (N - 1)], v[l], acc);
-      const int64_t o = base + q * stride;
-      T b = (T)0;
-      if (p.accumulate)
-        b = p.out[o];
-      else if (p.base)
-        b = p.base[o];
-      p.out[o] = fma(scale, acc, b);
-    }
-  } else {
+  {
     // the lines and the terms they are added to, all loads in flight before the arithmetic
     T v0[N], v1[N];
     float2 b[N];
@@ -102,7 +84,7 @@ __global__ void __launch_bounds__(128) k_kderiv(const KDerivParams<T, N> p) {
 // forms its line in registers, and the block stores the tile coalesced.
 template <typename T, int N>
 struct KDeriv3 {
-  static constexpr int LB = (sizeof(T) == 8 && N == 32) ? 64 : 128;   // lines per block
+  static constexpr int LB = 128;   // lines per block
 };
 
 // FP32 with N = 32: the tiles move as 16-byte quads (coalesced 512-byte warp accesses), quad q of
@@ -233,7 +215,7 @@ cudaError_t kderiv_tn(const Handle& H, const void* in, const void* base, void* o
       acc += (M_PI * m / H.g.lk) * std::sin(2.0 * M_PI * m * j / N);
     p.d[j] = (T)(-2.0 * acc / N);
   }
-  const unsigned nb = nblk(H.g.nxp * N * N / (sizeof(T) == 4 ? 2 : 1), 128);   // lines per thread
+  const unsigned nb = nblk(H.g.nxp * N * N / 2, 128);   // two lines per thread
   for (int d = 0; d < 3; ++d) {
     p.dim = d;
     p.accumulate = d > 0;
@@ -254,16 +236,20 @@ cudaError_t kderiv_tn(const Handle& H, const void* in, const void* base, void* o
 
 cudaError_t launch_theta_harm(const Handle& H, const void* in, const void* base, void* out,
                               double coef, cudaStream_t s) {
+  if (H.fp64) {
+    for (int d = 0; d < 3; ++d) {
+      const cudaError_t e = launch_kderiv_fx(H, in, d > 0 ? out : base, out, d, coef, s);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  }
   switch (H.g.nk) {
     case 8:
-      return H.fp64 ? kderiv_tn<double, 8>(H, in, base, out, coef, s)
-                    : kderiv_tn<float, 8>(H, in, base, out, coef, s);
+      return kderiv_tn<float, 8>(H, in, base, out, coef, s);
     case 16:
-      return H.fp64 ? kderiv_tn<double, 16>(H, in, base, out, coef, s)
-                    : kderiv_tn<float, 16>(H, in, base, out, coef, s);
+      return kderiv_tn<float, 16>(H, in, base, out, coef, s);
     case 32:
-      return H.fp64 ? kderiv_tn<double, 32>(H, in, base, out, coef, s)
-                    : kderiv_tn<float, 32>(H, in, base, out, coef, s);
+      return kderiv_tn<float, 32>(H, in, base, out, coef, s);
   }
   return cudaErrorInvalidValue;
 }

@@ -134,17 +134,16 @@ __global__ void k_moments_final(const double* __restrict__ partials, int nblocks
 // Quadratic potential: P(dt) is the exact shift f(x, k + s(x)), s_d = dt kappa (x_d - c_d)/hbar
 // (Eq. 5.1).  Per k-dimension it is the band-limited (periodic, spectral) shift, i.e. a circulant
 // matrix whose first column c[q] = (1/N) sum_m phi_m e^{2 pi i m q / N} is tabulated per x_d on
-// the host; one thread applies it to one k-line in registers.
+// the host; one thread applies it to its k-lines in registers (FP64: k_kpass_fx.cu).
 // ---------------------------------------------------------------------------------------------
-// FP64: one line per thread.  FP32: two lines per thread, k-adjacent in memory (r even and r + 1,
+// Two lines per thread, k-adjacent in memory (r even and r + 1,
 // the same x point), moved with 8-byte accesses, at three 128-thread CTAs per SM (a register bound
 // that spills a few coefficients but keeps 12 warps per SM: 6.25 -> 5.40 ms for the three passes
 // at 32^3 x 32^3).
 template <typename T, int N>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 3 : 1) k_kshift(T* __restrict__ f, int64_t nxp, int nx1, int nx2, int nx3, int dim,
+__global__ void __launch_bounds__(128, 3) k_kshift(T* __restrict__ f, int64_t nxp, int nx1, int nx2, int nx3, int dim,
                          const T* __restrict__ rows) {
-  constexpr int LPT = sizeof(T) == 4 ? 2 : 1;
-  const int64_t line = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * LPT;
+  const int64_t line = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 2;
   if (line >= nxp * N * N) return;
   const int64_t xp = line / (N * N);
   const int r = (int)(line % (N * N));
@@ -167,18 +166,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 3 : 1) k_kshift(T* __res
   T c[N];
 #pragma unroll
   for (int q = 0; q < N; ++q) c[q] = __ldg(crow + q);
-  if constexpr (LPT == 1) {
-    T v[N];
-#pragma unroll
-    for (int l = 0; l < N; ++l) v[l] = f[base + l * stride];
-#pragma unroll
-    for (int j = 0; j < N; ++j) {
-      T acc = (T)0;
-#pragma unroll
-      for (int l = 0; l < N; ++l) acc += c[(j - l + N) & (N - 1)] * v[l];
-      f[base + j * stride] = acc;
-    }
-  } else {
+  {
     T v0[N], v1[N];
 #pragma unroll
     for (int l = 0; l < N; ++l) {
@@ -453,27 +441,28 @@ cudaError_t launch_moments(const Handle& H, const void* f, double* partials, dou
 }
 
 cudaError_t launch_kshift(const Handle& H, void* f, int dim, const void* rows, cudaStream_t s) {
+  if (H.fp64) return launch_kshift_fx(H, f, dim, rows, H.d_kspec, s);
   const int64_t lines = H.g.nxp * H.g.nk * H.g.nk;
-  const unsigned nb = nblk(lines, 128), nb2 = nblk(lines / 2, 128);   // lines = nxp N^2 is even
+  const unsigned nb2 = nblk(lines / 2, 128);   // lines = nxp N^2 is even
   const int* nx = H.g.nx;
-#define CHASM_KS(TT, NN)                                                                           \
+#define CHASM_KS(NN)                                                                              \
   do {                                                                                             \
     if (dim == 2)                                                                                  \
-      k_kshift3<TT, NN><<<nblk(lines, kKsLines), kKsLines, 0, s>>>((TT*)f, H.g.nxp, nx[0], nx[1],  \
-                                                                   nx[2], (const TT*)rows);        \
+      k_kshift3<float, NN><<<nblk(lines, kKsLines), kKsLines, 0, s>>>((float*)f, H.g.nxp, nx[0],   \
+                                                                      nx[1], nx[2], (const float*)rows); \
     else                                                                                           \
-      k_kshift<TT, NN><<<sizeof(TT) == 4 ? nb2 : nb, 128, 0, s>>>((TT*)f, H.g.nxp, nx[0], nx[1],   \
-                                                                  nx[2], dim, (const TT*)rows);    \
+      k_kshift<float, NN><<<nb2, 128, 0, s>>>((float*)f, H.g.nxp, nx[0], nx[1], nx[2], dim,        \
+                                              (const float*)rows);                                 \
   } while (0)
   switch (H.g.nk) {
     case 8:
-      if (H.fp64) CHASM_KS(double, 8); else CHASM_KS(float, 8);
+      CHASM_KS(8);
       break;
     case 16:
-      if (H.fp64) CHASM_KS(double, 16); else CHASM_KS(float, 16);
+      CHASM_KS(16);
       break;
     case 32:
-      if (H.fp64) CHASM_KS(double, 32); else CHASM_KS(float, 32);
+      CHASM_KS(32);
       break;
     default:
       return cudaErrorInvalidValue;

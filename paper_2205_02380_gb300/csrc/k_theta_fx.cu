@@ -82,10 +82,6 @@ struct FxCfg {
   static_assert(NG * VSZ * sizeof(fxc) / NW >= 32 * TROW * 16, "line staging fits the slab buffers");
 };
 
-// magnitude bits to which the entries of a vector are aligned before a transform (the outputs of
-// two inverse halves are added: one bit less)
-constexpr int kFxBits = 57;
-
 // ---- barriers between the two warps of a group (mbarriers in shared memory) ----
 __device__ __forceinline__ unsigned sm_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mb_init(unsigned b, int warps) {
@@ -108,13 +104,6 @@ __device__ __forceinline__ bool mb_wait(unsigned b, int parity) {
   __syncwarp();
   return done != 0;
 }
-
-__device__ __forceinline__ void mag_or(unsigned& m, i64 x) {
-  const int h = (int)(x >> 32);
-  m |= (unsigned)(h ^ (h >> 31));
-}
-// number of bits that hold the magnitudes whose high words were or-ed into m
-__device__ __forceinline__ int mag_bits(unsigned m) { return 64 - __clz((int)m); }
 
 template <int N>
 __device__ __forceinline__ int seg_max(int v) {   // over the aligned groups of N lanes
@@ -150,17 +139,6 @@ __device__ __forceinline__ i64 ld_sym(const i64* p, uint64_t pol) {
 }
 __device__ __forceinline__ void prefetch_l2(const void* src, unsigned bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
-}
-
-// x y / 2^64 for a symbol value y in its stored form: high word, and the low word as a signed
-// number (the high word holds its carry)
-__device__ __forceinline__ i64 fx_mulsym(i64 x, i64 y) {
-  const int xh = (int)(x >> 32), yh = (int)(y >> 32), yl = (int)y;
-  const unsigned xl = (unsigned)x;
-  // the cross terms: signed high times unsigned low word (below 2^30 in magnitude: |yh| <= 2^30),
-  // and signed times signed (below 2^29.7)
-  const int t = (int)(__umulhi((unsigned)yh, xl) - (xl & (unsigned)(yh >> 31)) + (unsigned)__mulhi(yl, xh));
-  return fx_wide(xh, yh) + (i64)t;
 }
 
 // The lines of one warp (N doubles each, line of lane t at src + off(t)) into a staging buffer,
@@ -201,9 +179,6 @@ __device__ __forceinline__ void unstage_lines(double* dst, Off&& off, const doub
   __syncwarp();
 }
 
-// 2^e for e in [-900, 900]
-__device__ __forceinline__ double pow2_mid(int e) { return __hiloint2double((e + 1023) << 20, 0); }
-
 // The k3 twist e^{-i pi n / (2N)} of a real line (in shared memory), as integers with kFxBits
 // bits below the line's largest entry, whose exponent field is em; returns their exponent,
 // 1 << 30 when an entry is not finite.
@@ -213,13 +188,7 @@ __device__ __forceinline__ int quantise_line(const double* row, int em, fxc (&x)
     constexpr int n = decltype(I)::value;
     asm volatile("" ::: "memory");
     const double v = row[n];
-    const int hi = __double2hiint(v);
-    const int e = (hi >> 20) & 0x7ff;
-    const unsigned mh = (unsigned)(hi & 0xfffff) | (e ? 0x100000u : 0u);
-    u64 m = ((u64)mh << 32 | (unsigned)__double2loint(v)) << (kFxBits - 53);
-    m >>= min(63, em - max(e, 1));
-    const i64 sg = (i64)(hi >> 31);
-    const i64 w = ((i64)m ^ sg) - sg;
+    const i64 w = fx_from_double(v, em);
     if constexpr (n == 0) {
       x[n] = {w, 0};
     } else {
@@ -231,7 +200,7 @@ __device__ __forceinline__ int quantise_line(const double* row, int em, fxc (&x)
       x[n] = {fx_mul<c>(w), -fx_mul<s>(w)};
     }
   });
-  return em == 0x7ff ? 1 << 30 : em - 1023 - (kFxBits - 1);
+  return em == 0x7ff ? 1 << 30 : fx_exponent(em);
 }
 
 // sin phi Re z + cos phi Im z (the real part of -i e^{i phi} ... with the symbol's factor i taken
@@ -409,7 +378,7 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
           stage_lines<N, X2>(p.in, p.in2, p.cin2, off, S.T);
           em = 1;
 #pragma unroll
-          for (int n = 0; n < N; ++n) em = max(em, (__double2hiint(row[n]) >> 20) & 0x7ff);
+          for (int n = 0; n < N; ++n) em = max(em, fx_field(row[n]));
         }
         E = quantise_line<N>(row, em, x);
         if (E == 1 << 30) *S.flag = 1;
@@ -514,7 +483,7 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
           double th = (double)untwist<N, n, REAL>(x[n].im, x[n].re);
           if (em_ != E) th *= rest;
           const double v = fma(c2, th, row[n]);
-          em = max(em, (__double2hiint(v) >> 20) & 0x7ff);
+          em = max(em, fx_field(v));
           row[n] = v;
           asm volatile("" ::: "memory");   // one entry after the other: there are no registers to spare
         });

@@ -1,11 +1,13 @@
-"""Theta^T and P(dt) in double precision, whose transforms run in block fixed point: against the
-oracle at every N_k, exact under scaling by powers of two, with zero, tiny and non-finite data.
+"""Theta and P(dt) in double precision, Coulomb and quadratic, whose transforms run in block fixed
+point: against the oracle at every N_k, exact under scaling by powers of two, with zero, tiny and
+non-finite data.
 
 Tolerance against the oracle: a transform's entries carry 57 bits below the vector's largest
 entry and leave it about 3 units of the last one off, i.e. 2^-55; a padded vector's largest entry
 is at most 2^2.5 times its root mean square for the seeded data here; three forward and three
 inverse passes and the symbol product add up to under 8 2^-52.5 = 1.3e-15, and the oracle's own
-FFTs are off by about as much: 1e-14."""
+FFTs are off by about as much: 1e-14.  The quadratic passes transform each line twice per dimension:
+6 2^-54 and the oracle's part stay below it as well."""
 import numpy as np
 import pytest
 
@@ -91,5 +93,54 @@ def test_a_non_finite_entry_makes_its_x_point_nan_and_no_other(ch, nk, nx, value
         u[1, 2, 1, 3, 0, 5] = value
         got = _theta(s, torch.from_numpy(u).cuda())
     assert bool(torch.isnan(got[1, 2, 1]).all())
+    got[1, 2, 1] = want[1, 2, 1]
+    assert torch.equal(got, want)
+
+
+def _quadratic(ch, nx, nk):
+    return ch.Solver(nx, nk, LO, HI, LK, kappa=0.7, precision=ch.FP64)
+
+
+@pytest.mark.parametrize("nk,nx", GRIDS + [(32, (4, 4, 4)), (8, (7, 4, 9))])
+def test_quadratic_shift_and_derivative_match_the_oracle(ch, nk, nx):
+    u = _data(nx, nk, nk + 1)
+    prob = O.Problem(nx=nx, nk=nk, x_lo=LO, x_hi=HI, lk=LK, kappa=0.7)
+    with _quadratic(ch, nx, nk) as s:
+        d = torch.from_numpy(u).cuda()
+        assert O.rel_l2(_theta(s, d).cpu().numpy(), O.theta(u, prob)) <= TOL
+        s.pflow(d, 0.3)
+        s.sync()
+        assert O.rel_l2(d.cpu().numpy(), O.pflow(u, prob, 0.3)) <= TOL
+
+
+@pytest.mark.parametrize("nk,nx", GRIDS)
+def test_quadratic_lines_keep_their_own_scale(ch, nk, nx):
+    """Lines of neighbouring k3 are transformed together in the k1 and k2 passes: every second one
+    scaled by 2^300 comes out scaled (compared at the potential's centre in x_3, where k3 is not
+    shifted); scaling everything by a power of two is exact."""
+    u = torch.from_numpy(_data(nx, nk, 4)).cuda()
+    small = u * 2.0 ** -900
+    big = u.clone()
+    big[..., 1::2] *= 2.0 ** 300
+    c3 = (0.0, 0.0, LO[2])   # the first x_3 is the centre
+    with ch.Solver(nx, nk, LO, HI, LK, kappa=0.7, center=c3, precision=ch.FP64) as s:
+        for f in (u, small, big):
+            s.pflow(f, 0.3)
+    assert torch.equal(small, u * 2.0 ** -900)
+    got, want = big[:, :, 0], u[:, :, 0]
+    assert torch.allclose(got[..., 1::2] * 2.0 ** -300, want[..., 1::2], rtol=0, atol=1e-14)
+
+
+@pytest.mark.parametrize("nk,nx", GRIDS)
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+def test_a_non_finite_entry_of_the_quadratic_passes_stays_in_its_x_point(ch, nk, nx, value):
+    u = _data(nx, nk, 5)
+    with _quadratic(ch, nx, nk) as s:
+        want = torch.from_numpy(u).cuda()
+        s.pflow(want, 0.3)
+        u[1, 2, 1, 3, 0, 5] = value
+        got = torch.from_numpy(u).cuda()
+        s.pflow(got, 0.3)
+    assert not bool(torch.isfinite(got[1, 2, 1]).any())
     got[1, 2, 1] = want[1, 2, 1]
     assert torch.equal(got, want)
