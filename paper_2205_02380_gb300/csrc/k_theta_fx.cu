@@ -13,8 +13,9 @@
 // form issues in 40 % of the cycles (ncu at 640 x points, N_k = 32: integer pipe 40 %, multiplier
 // 35 %); two warps per scheduler, all that 64-bit vectors of 32 complex values leave registers
 // for, wait for their own results (1.06 warps per issue), for the L2-resident spectrum and the
-// symbol (0.60), and for instructions (0.56: 181 KB of code).  P(dt): 224.3 -> 37.3 ms at
-// 16^3 x 32^3, 77.7 -> 12.3 ms at 24^3 x 16^3.
+// symbol (0.60), and for instructions (0.56: 181 KB of code).  At N_k = 16 eight groups fit (all
+// slabs of an x point at once; four groups: 12.3 ms below).  P(dt): 224.3 -> 37.3 ms at
+// 16^3 x 32^3, 77.7 -> 11.0 ms at 24^3 x 16^3.
 //
 // Errors.  A vector enters a transform with 57 bits below its largest entry and leaves it with an
 // error of about 3 units of the last of them, so each of the eight transforms of a stage adds
@@ -67,7 +68,7 @@ template <int N>
 struct FxCfg {
   static constexpr int L = 2 * N;
   static constexpr int SPW = 32 / N;                 // slabs per group
-  static constexpr int NG = N == 8 ? 2 : 4;          // groups of two warps
+  static constexpr int NG = N == 8 ? 2 : (N == 16 ? 8 : 4);   // groups of two warps
   static constexpr int NT = 64 * NG;
   static constexpr int NW = NT / 32;
   static constexpr bool GSM = N <= 16;               // spectrum in shared memory
