@@ -4,34 +4,41 @@
 //   P(x1, x2)  = integral of f over x3 and k
 //   <x_d>, <k_d> = sum x_d f / sum f, sum k_d f / sum f   (averaged position and momentum)
 //
-// Stage 1 (k_diag_kpart, one launch per k-dimension d): S_d[x][q] = sum of f[x] over the two k
-// indices other than k_d = q, one thread per (x point, q), the other indices in row-major order.
-// Stage 2: W_j sums S_j over the other two x indices (thread per (x_j, q)); P sums S_0 over x3
-// and q (thread per (x1, x2)); the averages come from one block that reduces S_0, S_1, S_2 in a
-// fixed tree.  The grid factors (cell volumes, x and k node positions) are applied in FP64.
-#include "internal.hpp"
+// W_j and P: S_d[x][q] = sum of f[x] over the two k indices other than k_d = q (k_diag_kpart, f read
+// once), then W_j sums S_j over the other two x indices (a block per x_j) and P sums S_0 over x3
+// and q (a warp per (x1, x2)).  The averages read f once as well (k_diag_expect, the sums of
+// xsums.cuh); a second kernel adds the block partials in a fixed tree.  The grid factors (cell
+// volumes, x and k node positions) are applied in FP64.
+#include "xsums.cuh"
 
 namespace chasm {
 namespace {
 
 constexpr int kDiagThreads = 256;
 
-template <typename T, int N>
-__global__ void k_diag_kpart(const T* __restrict__ f, int64_t nxp, int d, double* __restrict__ S) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= nxp * N) return;
-  const int64_t xp = t / N;
-  const int q = (int)(t % N);
-  const T* fx = f + xp * (N * N * N);
+// Double precision: the same assignment as below with one value per access (the FP64 pipe adds 1.7
+// per clock and SM, which one 8-byte access per lane keeps up with): D = 0, 1 a warp per (x
+// point, q), D = 2 a warp per x point with one k3 per lane.
+template <int N, int D>
+__global__ void __launch_bounds__(kDiagThreads) k_diag_kpart_d(const double* __restrict__ f, int64_t nxp,
+                                                               double* __restrict__ S) {
+  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (w >= (D < 2 ? nxp * N : nxp)) return;
+  const int q = (int)(w % N);
+  const double* base = f + (D < 2 ? w / N : w) * (N * N * N);
+  constexpr int kEach = D < 2 ? N * N : N * N * N;
   double s = 0.0;
-  for (int a = 0; a < N; ++a) {
 #pragma unroll 8
-    for (int b = 0; b < N; ++b) {
-      const int off = d == 0 ? (q * N + a) * N + b : (d == 1 ? (a * N + q) * N + b : (a * N + b) * N + q);
-      s += (double)fx[off];
-    }
+  for (int g = lane; g < kEach; g += 32)
+    s += __ldcs(base + (D == 0 ? q * N * N + g : (D == 1 ? (g / N * N + q) * N + g % N : g)));
+#pragma unroll
+  for (int o = D < 2 ? 1 : N; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if constexpr (D < 2) {
+    if (lane == 0) S[w] = s;
+  } else {
+    if (lane < N) S[w * N + lane] = s;
   }
-  S[t] = s;
 }
 
 // Single precision: one warp per (x point, q) for d = 0, 1 and one warp per x point for d = 2,
@@ -97,13 +104,14 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_kpart_w(const float* __re
 // W_j[i][q] = vol * sum over the other two x indices of S_j[x][q]: one block per i, thread t adds
 // q = t mod N over the (a, b) pairs t / N, t / N + G, ... (G = threads / N), then the G partials
 // of each q in ascending order (a fixed order: bitwise reproducible)
-__global__ void __launch_bounds__(kDiagThreads) k_diag_wigner(const double* __restrict__ S, int j, int nx0,
-                                                              int nx1, int nx2, int N, double vol,
-                                                              double* __restrict__ W) {
-  __shared__ double part[kDiagThreads];
+constexpr int kWigThreads = 1024;   // one block per x_j: few blocks, so wide ones (256 threads: 43 us at 32^3)
+__global__ void __launch_bounds__(kWigThreads) k_diag_wigner(const double* __restrict__ S, int j, int nx0,
+                                                             int nx1, int nx2, int N, double vol,
+                                                             double* __restrict__ W) {
+  __shared__ double part[kWigThreads];
   const int nx[3] = {nx0, nx1, nx2};
   const int i = blockIdx.x, t = threadIdx.x;
-  const int q = t % N, G = kDiagThreads / N;
+  const int q = t % N, G = kWigThreads / N;
   const int oa = j == 0 ? 1 : 0, ob = j == 2 ? 1 : 2;
   double s = 0.0;
   for (int ab = t / N; ab < nx[oa] * nx[ob]; ab += G) {
@@ -123,66 +131,75 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_wigner(const double* __re
   }
 }
 
-// P[i1][i2] = vol * sum over i3 and q of S_0[x][q]
+// P[i1][i2] = vol * sum over i3 and q of S_0[x][q]: one warp per (i1, i2) (a thread each: 161 us at
+// 32^3 x 32^3)
 __global__ void k_diag_marginal(const double* __restrict__ S0, int nx0, int nx1, int nx2, int N,
                                 double vol, double* __restrict__ P) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int t = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   if (t >= nx0 * nx1) return;
+  const int lane = threadIdx.x & 31;
+  const double* r = S0 + (int64_t)t * nx2 * N;
   double s = 0.0;
-  for (int i3 = 0; i3 < nx2; ++i3) {
-    const double* r = S0 + ((int64_t)t * nx2 + i3) * N;
-    for (int q = 0; q < N; ++q) s += r[q];
-  }
-  P[t] = s * vol;
+#pragma unroll 8
+  for (int e = lane; e < nx2 * N; e += 32) s += r[e];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) P[t] = s * vol;
 }
 
-// Averages, stage 1 (kExpBlocks blocks, each a fixed range of x points): m = sum S_0,
-// x_d m, k_d = sum_q k_q S_d; the 7 block partials go to part[7 * block + c]
-constexpr int kExpBlocks = 256;
-__global__ void __launch_bounds__(kDiagThreads) k_diag_expect(const double* __restrict__ S, int64_t nxp,
-                                                              int nx1, int nx2, int N, double3 xlo,
-                                                              double3 h, double dk,
-                                                              double* __restrict__ part) {
-  __shared__ double red[7][kDiagThreads];
-  const int tid = threadIdx.x;
+// Averages: per block the sums of f, of i_d f (x index) and of k_d f (integer k) over its x points.  Three reads
+// of f, one per k-dimension, took 1.75 ms at 32^3 x 32^3 FP32, this one 0.78.
+// fixed: the order of the sums does not depend on the device; four blocks on each of 152 SMs
+constexpr int kExpBlocks = 608;
+template <typename T, int N>
+__global__ void __launch_bounds__(XSums<T, N>::kThreads) k_diag_expect(const T* __restrict__ f, int64_t nxp,
+                                                                       int nx1, int nx2, bool wide,
+                                                                       double* __restrict__ part) {
+  using X = XSums<T, N>;
+  const X me;
   double acc[7] = {0, 0, 0, 0, 0, 0, 0};
-  const int64_t per = (nxp + gridDim.x - 1) / gridDim.x;
-  const int64_t x0 = (int64_t)blockIdx.x * per, x1 = min(nxp, x0 + per);
-  for (int64_t xp = x0 + tid; xp < x1; xp += kDiagThreads) {
-    const int i3 = (int)(xp % nx2), i2 = (int)((xp / nx2) % nx1), i1 = (int)(xp / ((int64_t)nx1 * nx2));
-    double m = 0.0, k[3] = {0, 0, 0};
-    for (int q = 0; q < N; ++q) {
-      const double kq = (q - N / 2) * dk;
-      m += S[xp * N + q];
-      for (int d = 0; d < 3; ++d) k[d] += kq * S[((int64_t)d * nxp + xp) * N + q];
+  Run<T> run[7];
+  int n = 0;
+  for (int64_t xp = blockIdx.x; xp < nxp; xp += gridDim.x) {
+    // an x point holds at least 2 KB, so their number fits 32 bits
+    const unsigned x = (unsigned)xp, r = x / (unsigned)nx2;
+    const int i3 = (int)(x % (unsigned)nx2), i2 = (int)(r % (unsigned)nx1), i1 = (int)(r / (unsigned)nx1);
+    Run<T> m, u, v;
+    me.template add<false>(f + xp * (N * N * N), wide, m, u, v);
+    run[0].add(m);
+    run[1].add(m, (float)i1);
+    run[2].add(m, (float)i2);
+    run[3].add(m, (float)i3);
+    run[4].add(u);
+    run[5].add(m, (float)me.k2);
+    run[6].add(v);
+    if (++n == kRunLength<T> || xp + gridDim.x >= nxp) {
+#pragma unroll
+      for (int c = 0; c < 7; ++c) acc[c] += run[c].take();
+      n = 0;
     }
-    acc[0] += m;
-    acc[1] += (xlo.x + i1 * h.x) * m;
-    acc[2] += (xlo.y + i2 * h.y) * m;
-    acc[3] += (xlo.z + i3 * h.z) * m;
-    for (int d = 0; d < 3; ++d) acc[4 + d] += k[d];
   }
-  for (int c = 0; c < 7; ++c) red[c][tid] = acc[c];
-  __syncthreads();
-  for (int s = kDiagThreads / 2; s > 0; s >>= 1) {
-    if (tid < s)
-      for (int c = 0; c < 7; ++c) red[c][tid] += red[c][tid + s];
-    __syncthreads();
-  }
-  if (tid == 0)
-    for (int c = 0; c < 7; ++c) part[7 * blockIdx.x + c] = red[c][0];
+  block_sum_store<7>(acc, part);
 }
 
-// Averages, stage 2 (one thread per average): the block partials in ascending order
-__global__ void k_diag_expect_final(const double* __restrict__ part, int nb, double* __restrict__ out) {
+// the block partials in a fixed tree; out[d] = x_lo + h sum i_d f / sum f, out[3 + d] = dk sum k_d f /
+// sum f
+__global__ void __launch_bounds__(kDiagThreads) k_diag_expect_final(const double* __restrict__ part, int nb,
+                                                                    double3 xlo, double3 h, double dk,
+                                                                    double* __restrict__ out) {
+  __shared__ double tot[7];
+  double v[7] = {0, 0, 0, 0, 0, 0, 0};
+  for (int b = threadIdx.x; b < nb; b += kDiagThreads)
+#pragma unroll
+    for (int c = 0; c < 7; ++c) v[c] += part[7 * b + c];
+  block_sum_store<7>(v, tot);
+  __syncthreads();
   const int c = threadIdx.x;
-  if (c >= 6) return;
-  double m = 0.0, v = 0.0;
-  for (int b = 0; b < nb; ++b) {
-    m += part[7 * b];
-    v += part[7 * b + 1 + c];
+  if (c < 6) {
+    const double lo = c == 0 ? xlo.x : (c == 1 ? xlo.y : (c == 2 ? xlo.z : 0.0));
+    const double step = c == 0 ? h.x : (c == 1 ? h.y : (c == 2 ? h.z : dk));
+    out[c] = fma(step, tot[1 + c] / tot[0], lo);
   }
-  out[c] = v / m;
 }
 
 inline unsigned nblk(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
@@ -197,9 +214,24 @@ cudaError_t kpart_tn(const Handle& H, const void* f, int d, double* S, cudaStrea
     if (d == 0) k_diag_kpart_w<N, 0><<<nb, kDiagThreads, 0, s>>>(ff, H.g.nxp, Sd);
     else if (d == 1) k_diag_kpart_w<N, 1><<<nb, kDiagThreads, 0, s>>>(ff, H.g.nxp, Sd);
     else k_diag_kpart_w<N, 2><<<nb, kDiagThreads, 0, s>>>(ff, H.g.nxp, Sd);
-  } else
-    k_diag_kpart<T, N><<<nblk(H.g.nxp * N, kDiagThreads), kDiagThreads, 0, s>>>(
-        static_cast<const T*>(f), H.g.nxp, d, S + (size_t)d * H.g.nxp * N);
+  } else {
+    const double* fd = static_cast<const double*>(f);
+    double* Sd = S + (size_t)d * H.g.nxp * N;
+    const unsigned nb = nblk((d == 2 ? H.g.nxp : H.g.nxp * N) * 32, kDiagThreads);
+    if (d == 0) k_diag_kpart_d<N, 0><<<nb, kDiagThreads, 0, s>>>(fd, H.g.nxp, Sd);
+    else if (d == 1) k_diag_kpart_d<N, 1><<<nb, kDiagThreads, 0, s>>>(fd, H.g.nxp, Sd);
+    else k_diag_kpart_d<N, 2><<<nb, kDiagThreads, 0, s>>>(fd, H.g.nxp, Sd);
+  }
+  return cudaGetLastError();
+}
+
+template <typename T, int N>
+cudaError_t expect_tn(const Handle& H, const void* f, double* part, double* out, cudaStream_t s) {
+  const int nb = (int)std::min<int64_t>(kExpBlocks, H.g.nxp);
+  k_diag_expect<T, N><<<nb, XSums<T, N>::kThreads, 0, s>>>(
+      static_cast<const T*>(f), H.g.nxp, H.g.nx[1], H.g.nx[2], (reinterpret_cast<uintptr_t>(f) & 15) == 0, part);
+  k_diag_expect_final<<<1, kDiagThreads, 0, s>>>(part, nb, make_double3(H.g.x_lo[0], H.g.x_lo[1], H.g.x_lo[2]),
+                                                 make_double3(H.g.h[0], H.g.h[1], H.g.h[2]), H.g.dk, out);
   return cudaGetLastError();
 }
 
@@ -231,23 +263,22 @@ cudaError_t launch_diag(const Handle& H, const void* f, int what, int j, double*
     if (e != cudaSuccess) return e;
     const int oa = j == 0 ? 1 : 0, ob = j == 2 ? 1 : 2;
     const double vol = H.g.h[oa] * H.g.h[ob] * H.g.dk * H.g.dk;
-    k_diag_wigner<<<nx[j], kDiagThreads, 0, s>>>(buf + (size_t)j * H.g.nxp * N, j, nx[0], nx[1],
+    k_diag_wigner<<<nx[j], kWigThreads, 0, s>>>(buf + (size_t)j * H.g.nxp * N, j, nx[0], nx[1],
                                                  nx[2], N, vol, out_dev);
   } else if (what == 1) {   // marginal P(x1, x2)
     e = kpart(H, f, 0, buf, s);
     if (e != cudaSuccess) return e;
     const double vol = H.g.h[2] * H.g.dk * H.g.dk * H.g.dk;
-    k_diag_marginal<<<nblk((int64_t)nx[0] * nx[1], kDiagThreads), kDiagThreads, 0, s>>>(
+    k_diag_marginal<<<nblk((int64_t)nx[0] * nx[1] * 32, kDiagThreads), kDiagThreads, 0, s>>>(
         buf, nx[0], nx[1], nx[2], N, vol, out_dev);
   } else {   // averages
-    for (int d = 0; d < 3 && e == cudaSuccess; ++d) e = kpart(H, f, d, buf, s);
-    if (e != cudaSuccess) return e;
-    // the block partials go behind the six results (diag_bytes reserves them)
-    double* part = out_dev + 8;
-    k_diag_expect<<<kExpBlocks, kDiagThreads, 0, s>>>(buf, H.g.nxp, nx[1], nx[2], N,
-                                                      make_double3(H.g.x_lo[0], H.g.x_lo[1], H.g.x_lo[2]),
-                                                      make_double3(H.g.h[0], H.g.h[1], H.g.h[2]), H.g.dk, part);
-    k_diag_expect_final<<<1, 32, 0, s>>>(part, kExpBlocks, out_dev);
+    double* part = out_dev + 8;   // the block partials go behind the six results (diag_bytes reserves them)
+    switch (N) {
+      case 8: return H.fp64 ? expect_tn<double, 8>(H, f, part, out_dev, s) : expect_tn<float, 8>(H, f, part, out_dev, s);
+      case 16: return H.fp64 ? expect_tn<double, 16>(H, f, part, out_dev, s) : expect_tn<float, 16>(H, f, part, out_dev, s);
+      case 32: return H.fp64 ? expect_tn<double, 32>(H, f, part, out_dev, s) : expect_tn<float, 32>(H, f, part, out_dev, s);
+    }
+    return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
 }

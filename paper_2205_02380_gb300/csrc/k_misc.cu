@@ -2,102 +2,39 @@
 #include <algorithm>
 #include <cmath>
 
-#include "internal.hpp"
+#include "xsums.cuh"
 
 namespace chasm {
 namespace {
 
-constexpr int kMomBlocks = 1024;   // fixed: the reduction tree does not depend on the device
+// fixed: the reduction tree does not depend on the device; four blocks on each of 152 SMs, one wave
+constexpr int kMomBlocks = 608;
 constexpr int kMomThreads = 256;
 
 // ---------------------------------------------------------------------------------------------
 // Mass and energy (diagnostics of Sec. 5): per x point, S0 = sum_k f and S2 = sum_k |k|^2 f;
 // mass += S0, energy += (hbar^2/2m) dk^2 S2' + V(x) S0 where S2' uses integer |j - N/2|^2.
-// Every thread accumulates its own elements of the block's x points (V(x) S0 is linear in the
-// thread's partial of S0, so no per-x-point reduction is needed); one block reduction at the end
-// and a second kernel that adds the block partials in a fixed order make the result bitwise
-// reproducible (the grid size is fixed).
+// Every thread adds up its own elements of the block's x points (xsums.cuh; V(x) S0 is linear in
+// the thread's part of S0, so nothing is reduced per x point); one block reduction at the end and
+// a second kernel that adds the block partials in a fixed order make the result bitwise
+// reproducible (the grid size is fixed).  32^3 x 32^3 FP32: 818 us with the whole weight formed per
+// element and 1024 blocks, 711 us with the weights of k2 and k3 applied per x point and one wave of
+// blocks (HBM alone 632 us).
 // ---------------------------------------------------------------------------------------------
-template <int NV>
-__device__ __forceinline__ void block_sum_store(double (&v)[NV], double* __restrict__ out) {
-  __shared__ double red[NV][kMomThreads / 32];
-  const int tid = threadIdx.x;
-#pragma unroll
-  for (int c = 0; c < NV; ++c)
-    for (int o = 16; o > 0; o >>= 1) v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
-  if ((tid & 31) == 0)
-#pragma unroll
-    for (int c = 0; c < NV; ++c) red[c][tid >> 5] = v[c];
-  __syncthreads();
-  if (tid == 0)
-#pragma unroll
-    for (int c = 0; c < NV; ++c) {
-      double a = 0.0;
-      for (int w = 0; w < kMomThreads / 32; ++w) a += red[c][w];
-      out[(int64_t)NV * blockIdx.x + c] = a;
-    }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kMomThreads) k_moments(const T* __restrict__ f, int64_t nxp,
-                                                         int nk, const double* __restrict__ vx,
-                                                         double* __restrict__ partials) {
-  const int kvol = nk * nk * nk;
+template <typename T, int N>
+__global__ void __launch_bounds__(XSums<T, N>::kThreads) k_moments(const T* __restrict__ f, int64_t nxp,
+                                                                   const double* __restrict__ vx, bool wide,
+                                                                   double* __restrict__ partials) {
+  using X = XSums<T, N>;
+  const X me;
   double acc[3] = {0.0, 0.0, 0.0};   // sum f, sum |j - N/2|^2 f, sum V(x) f
   for (int64_t xp = blockIdx.x; xp < nxp; xp += gridDim.x) {
-    const T* fx = f + xp * kvol;
-    double s0 = 0.0, s2 = 0.0;
-    for (int e = threadIdx.x; e < kvol; e += kMomThreads) {
-      const double v = (double)fx[e];
-      const int k3 = e % nk - nk / 2, k2 = (e / nk) % nk - nk / 2, k1 = e / (nk * nk) - nk / 2;
-      s0 += v;
-      s2 += v * (double)(k1 * k1 + k2 * k2 + k3 * k3);
-    }
+    Run<T> m, u, none;
+    me.template add<true>(f + xp * (N * N * N), wide, m, u, none);
+    const double s0 = m.take();
     acc[0] += s0;
-    acc[1] += s2;
-    acc[2] += vx[xp] * s0;
-  }
-  block_sum_store<3>(acc, partials);
-}
-
-// Single precision: the FP64 pipe (1/64 of the FP32 rate on this part) cannot keep up with one
-// FP64 add per element at HBM speed, so each thread sums its elements of an x point in compensated
-// FP32 pairs (Knuth's error-free two-sum; the products v |k|^2 with their exact FMA residual; about
-// 2^-44 relative) and adds the pairs to FP64 accumulators once per x point; float4 loads, eight in
-// flight per thread.
-template <>
-__global__ void __launch_bounds__(kMomThreads) k_moments<float>(const float* __restrict__ f, int64_t nxp,
-                                                                int nk, const double* __restrict__ vx,
-                                                                double* __restrict__ partials) {
-  const int tid = threadIdx.x;
-  const int lg = __ffs(nk) - 1;              // nk is a power of two
-  const int kvol4 = (nk * nk * nk) >> 2;     // float4 per x point
-  const int half = nk >> 1;
-  double acc[3] = {0.0, 0.0, 0.0};
-  for (int64_t xp = blockIdx.x; xp < nxp; xp += gridDim.x) {
-    const float4* fx = reinterpret_cast<const float4*>(f + xp * (int64_t)(kvol4 << 2));
-    float h0 = 0.f, l0 = 0.f, h2 = 0.f, l2 = 0.f;
-#pragma unroll 8
-    for (int e4 = tid; e4 < kvol4; e4 += kMomThreads) {
-      const float4 q = __ldcs(fx + e4);
-      const float v[4] = {q.x, q.y, q.z, q.w};
-      const int e = e4 << 2;
-      const int k1 = (e >> (2 * lg)) - half, k2 = ((e >> lg) & (nk - 1)) - half;
-      const int k3b = (e & (nk - 1)) - half;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int k3 = k3b + c;
-        const float w = (float)(k1 * k1 + k2 * k2 + k3 * k3);   // exact: at most 3 (nk/2)^2
-        two_sum_f(h0, l0, v[c]);
-        const float pr = v[c] * w;
-        l2 += fmaf(v[c], w, -pr);                                 // exact product residual
-        two_sum_f(h2, l2, pr);
-      }
-    }
-    const double s0 = (double)h0 + (double)l0;
-    acc[0] += s0;
-    acc[1] += (double)h2 + (double)l2;
-    acc[2] += vx[xp] * s0;
+    acc[1] += u.take();
+    acc[2] = fma(vx[xp], s0, acc[2]);
   }
   block_sum_store<3>(acc, partials);
 }
@@ -430,10 +367,23 @@ int moments_blocks() { return kMomBlocks; }
 cudaError_t launch_moments(const Handle& H, const void* f, double* partials, double* result_dev,
                            cudaStream_t s) {
   const int nb = (int)std::min<int64_t>(kMomBlocks, H.g.nxp);
-  if (H.fp64)
-    k_moments<double><<<nb, kMomThreads, 0, s>>>((const double*)f, H.g.nxp, H.g.nk, H.d_vx, partials);
-  else
-    k_moments<float><<<nb, kMomThreads, 0, s>>>((const float*)f, H.g.nxp, H.g.nk, H.d_vx, partials);
+  const bool wide = (reinterpret_cast<uintptr_t>(f) & 15) == 0;
+#define CHASM_MOM(TT, NN) \
+  k_moments<TT, NN><<<nb, XSums<TT, NN>::kThreads, 0, s>>>((const TT*)f, H.g.nxp, H.d_vx, wide, partials)
+  switch (H.g.nk) {
+    case 8:
+      if (H.fp64) CHASM_MOM(double, 8); else CHASM_MOM(float, 8);
+      break;
+    case 16:
+      if (H.fp64) CHASM_MOM(double, 16); else CHASM_MOM(float, 16);
+      break;
+    case 32:
+      if (H.fp64) CHASM_MOM(double, 32); else CHASM_MOM(float, 32);
+      break;
+    default:
+      return cudaErrorInvalidValue;
+  }
+#undef CHASM_MOM
   const double cell = H.g.h[0] * H.g.h[1] * H.g.h[2] * H.g.dk * H.g.dk * H.g.dk;
   const double kin = H.hbar * H.hbar / (2.0 * H.m) * H.g.dk * H.g.dk;
   k_moments_final<<<1, kMomThreads, 0, s>>>(partials, nb, cell, kin, result_dev);
