@@ -429,96 +429,108 @@ struct PatchArgs {
   const T* lu;    // [c' (M+1) | 1/pivot (M+1)] of the (M+1)-node patch system
 };
 
-// closure value of boundary b = sum over its window of coefficient * phi, hi/lo parts
+// closure value of boundary b = sum over its window of coefficient * phi, hi/lo parts; phi_j at
+// buf[j B], taps outside [0, N] dropped
 __device__ __forceinline__ void patch_closure(const PatchArgs<double>& q, const double* buf, int B, int N,
                                               int b, double& hi, double& lo) {
+  const int first = b * q.M - q.nb, i0 = max(0, -first), i1 = min(q.W - 1, N - first);
+  const double* w = q.win + (size_t)b * q.W;
   double acc = 0.0;
-  for (int i = 0; i < q.W; ++i) {
-    const int node = b * q.M - q.nb + i;
-    if (node >= 0 && node <= N) acc = fma(__ldg(q.win + (size_t)b * q.W + i), buf[(size_t)node * B], acc);
-  }
+#pragma unroll 4
+  for (int i = i0; i <= i1; ++i) acc = fma(__ldg(w + i), buf[(first + i) * B], acc);
   hi = acc;
   lo = 0.0;
 }
 __device__ __forceinline__ void patch_closure(const PatchArgs<float>& q, const float* buf, int B, int N,
                                               int b, float& hi, float& lo) {
-  DF acc{0.f, 0.f};
+  const int first = b * q.M - q.nb, i0 = max(0, -first), i1 = min(q.W - 1, N - first);
   const float* w = q.win + (size_t)b * 2 * q.W;
-  for (int i = 0; i < q.W; ++i) {
-    const int node = b * q.M - q.nb + i;
-    if (node >= 0 && node <= N) df_acc(acc, buf[(size_t)node * B], __ldg(w + i), __ldg(w + q.W + i));
-  }
+  DF acc{0.f, 0.f};
+#pragma unroll 4
+  for (int i = i0; i <= i1; ++i) df_acc(acc, buf[(first + i) * B], __ldg(w + i), __ldg(w + q.W + i));
   hi = acc.hi;
   lo = acc.lo;
 }
 
+// All closures are formed first; then each patch is solved in place over its nodes and evaluated
+// before the next one starts, so a line needs n + 2 values and its closures: the left ghost takes
+// the slot before the patch (done with), the right ghost borrows the slot behind it, and the node
+// two patches share is handed on.  With every patch's coefficients kept, 121 points in 4 patches
+// left room for 3 FP64 warps per SM, which cannot keep the four FP64 pipes busy: 4.15 -> 2.03 ms a pass
+// at 121 x 5^2 x 32^3 (6 warps).
 template <typename T>
 __global__ void __launch_bounds__(kAdvectThreads) k_advect_patches(AdvParams<T> p, PatchArgs<T> q) {
+  constexpr int kParts = sizeof(T) == 4 ? 2 : 1;            // hi and lo part of a closure
   extern __shared__ unsigned char smem_raw[];
   const int B = blockDim.x;
   const int n = p.n, N = n - 1, P = q.P, M = q.M;
-  T* buf = reinterpret_cast<T*>(smem_raw) + threadIdx.x;   // phi_j at buf[j B]
-  T* cvh = buf + (size_t)n * B;                             // closure b: cvh[b B], cvl[b B]
-  T* cvl = cvh + (size_t)(P + 1) * B;
-  T* eta = cvl + (size_t)(P + 1) * B;                       // eta^(l)_nu at eta[(l (M+3) + nu + 1) B]
+  T* buf = reinterpret_cast<T*>(smem_raw) + threadIdx.x + B;   // phi_j at buf[j B], j = -1..n
+  T* cv = buf + (n + 1) * B;                                    // closure b at cv[kParts b B] (and + B)
   const int64_t line = (int64_t)blockIdx.x * B + threadIdx.x;
-  if (line >= p.n_lines) return;
+  if (line >= p.n_lines) return;                                // whole warps: kvol is a multiple of 32
   T* src;
   int kd;
   line_setup(p, line, src, kd);
-  for (int j = 0; j < n; ++j) buf[(size_t)j * B] = src[(int64_t)j * p.s_d];
+#pragma unroll 8
+  for (int j = 0; j < n; ++j) buf[j * B] = src[(int64_t)j * p.s_d];
   for (int b = 0; b <= P; ++b) {
     T hi, lo;
     patch_closure(q, buf, B, N, b, hi, lo);
-    cvh[(size_t)b * B] = hi;
-    cvl[(size_t)b * B] = lo;
+    cv[kParts * b * B] = hi;
+    if constexpr (kParts == 2) cv[(2 * b + 1) * B] = lo;
   }
   const T* cprime = q.lu;
   const T* mult = q.lu + (M + 1);
-  for (int l = 0; l < P; ++l) {
-    const T* ph = buf + (size_t)l * M * B;
-    T* e = eta + (size_t)l * (M + 3) * B;
-    Closure<T> cl;   // phi_L of patch l in cl.L, phi_R in cl.R
-    if constexpr (sizeof(T) == 4) {
-      cl.L = DF{cvh[(size_t)l * B], cvl[(size_t)l * B]};
-      cl.R = DF{cvh[(size_t)(l + 1) * B], cvl[(size_t)(l + 1) * B]};
-    } else {
-      cl.L = cvh[(size_t)l * B];
-      cl.R = cvh[(size_t)(l + 1) * B];
-    }
-    T dp = (T)cl.d0(ph[0], hval(p)) * __ldg(mult);
-    e[B] = dp;
-    for (int i = 1; i < M; ++i) {
-      dp = ((T)6 * ph[(size_t)i * B] - dp) * __ldg(mult + i);
-      e[(size_t)(i + 1) * B] = dp;
-    }
-    dp = ((T)cl.dN(ph[(size_t)M * B], hval(p)) - dp) * __ldg(mult + M);
-    e[(size_t)(M + 1) * B] = dp;
-    T nx = dp;
-    for (int i = M - 1; i >= 0; --i) {
-      nx = e[(size_t)(i + 1) * B] - __ldg(cprime + i) * nx;
-      e[(size_t)(i + 1) * B] = nx;
-    }
-    e[0] = (T)cl.gl(e[2 * (size_t)B], h2val(p));
-    e[(size_t)(M + 2) * B] = (T)cl.gr(e[(size_t)M * B], h2val(p));
-  }
   const int sh = __ldg(p.ns + kd);
   const T w[4] = {__ldg(p.w + 4 * kd + 0), __ldg(p.w + 4 * kd + 1), __ldg(p.w + 4 * kd + 2),
                   __ldg(p.w + 4 * kd + 3)};
-  for (int j = 0; j < n; ++j) {
-    // patch of the foot x_j - (sh + a) h: floor((j - sh - 1) / M), clamped (left patch at a node)
-    const int t = j - sh - 1;
-    int l = t >= 0 ? t / M : -((-t + M - 1) / M);
-    l = l < 0 ? 0 : (l > P - 1 ? P - 1 : l);
-    const int nu0 = j - l * M - sh - 2;   // first tap, local index
-    const T* e = eta + (size_t)l * (M + 3) * B;
-    T acc = (T)0;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int nu = nu0 + c;
-      if (nu >= -1 && nu <= M + 1) acc = fma(w[c], e[(size_t)(nu + 1) * B], acc);
+  T shared = buf[0];   // phi at the patch's first node
+  for (int l = 0; l < P; ++l) {
+    T* e = buf + l * M * B;   // eta_nu of this patch at e[nu B], nu = -1..M+1
+    Closure<T> cl;            // phi_L of patch l in cl.L, phi_R in cl.R
+    if constexpr (kParts == 2) {
+      cl.L = DF{cv[2 * l * B], cv[(2 * l + 1) * B]};
+      cl.R = DF{cv[(2 * l + 2) * B], cv[(2 * l + 3) * B]};
+    } else {
+      cl.L = cv[l * B];
+      cl.R = cv[(l + 1) * B];
     }
-    src[(int64_t)j * p.s_d] = acc;
+    const T behind = e[(M + 1) * B], last = e[M * B];
+    T dp = (T)cl.d0(shared, hval(p)) * __ldg(mult);
+    e[0] = dp;
+#pragma unroll 4
+    for (int i = 1; i < M; ++i) {
+      dp = ((T)6 * e[i * B] - dp) * __ldg(mult + i);
+      e[i * B] = dp;
+    }
+    dp = ((T)cl.dN(last, hval(p)) - dp) * __ldg(mult + M);
+    e[M * B] = dp;
+    T nx = dp;
+#pragma unroll 4
+    for (int i = M - 1; i >= 0; --i) {
+      nx = e[i * B] - __ldg(cprime + i) * nx;
+      e[i * B] = nx;
+    }
+    e[-B] = (T)cl.gl(e[B], h2val(p));
+    e[(M + 1) * B] = (T)cl.gr(e[(M - 1) * B], h2val(p));
+    // the nodes whose foot x_j - (sh + a) h lies in this patch (the left patch at a shared node, the
+    // end patches beyond the ends): j - sh - 1 in [l M, (l + 1) M); one loop for the warp
+    const int j0 = l == 0 ? 0 : max(0, l * M + sh + 1);
+    const int j1 = l == P - 1 ? n - 1 : min(n - 1, l * M + M + sh);
+    const int first = __reduce_min_sync(0xffffffffu, j0), final = __reduce_max_sync(0xffffffffu, j1);
+#pragma unroll 4
+    for (int j = first; j <= final; ++j) {
+      const int nu0 = j - l * M - sh - 2;   // first tap, local index
+      T acc = (T)0;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int nu = nu0 + c;
+        if (nu >= -1 && nu <= M + 1) acc = fma(w[c], e[nu * B], acc);
+      }
+      if (j >= j0 && j <= j1) src[(int64_t)j * p.s_d] = acc;
+    }
+    e[(M + 1) * B] = behind;
+    shared = last;
   }
 }
 
@@ -620,8 +632,19 @@ cudaError_t launch_t(const Handle& H, void* f, int dim, cudaStream_t s) {
     q.W = 2 * q.nb + 1;
     q.win = static_cast<const T*>(H.d_pclos[dim]);
     q.lu = static_cast<const T*>(H.d_plu[dim]);
-    const size_t elems = advect_smem_elems(p.n, P);
-    const int Bp = advect_smem_threads(elems, sizeof(T));
+    const size_t elems = (size_t)p.n + 2 + (size_t)(P + 1) * (sizeof(T) == 4 ? 2 : 1);
+    // the block size that leaves the most threads on an SM
+    int Bp = 0;
+    size_t most = 0;
+    for (int b = kAdvectThreads; b >= 32; b -= 32) {
+      const size_t bytes = elems * b * sizeof(T);
+      if (bytes > (size_t)kAdvectMaxSmem) continue;
+      const size_t on = (size_t)(227 * 1024) / (bytes + 1024) * b;
+      if (on > most) {
+        most = on;
+        Bp = b;
+      }
+    }
     if (Bp == 0) return cudaErrorInvalidValue;
     k_advect_patches<T><<<(unsigned)((p.n_lines + Bp - 1) / Bp), Bp, elems * Bp * sizeof(T), s>>>(p, q);
     return cudaGetLastError();
