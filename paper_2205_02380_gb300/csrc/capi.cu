@@ -326,6 +326,38 @@ static void round_unit_sum(const double* w, float* out, int n) {
   out[jmin] = (float)(1.0 - rest);
 }
 
+// The pass along dimension d as an n x n matrix per k (k_advect_dense): closure, solve and 4-tap
+// evaluation with the plan's stencils and factors applied to unit vectors; w, ns: the weights and
+// shifts of the nk values of k; out[(j n + q) nk + k].
+static void dense_rows(const Handle* H, int d, const double* w, const int* ns, double* out) {
+  const int n = H->g.nx[d], N = n - 1, nk = H->g.nk;
+  const double h = H->g.h[d];
+  const std::vector<double>&c = H->h_clos[d], &lu = H->h_lu[d];
+  for (int q = 0; q < n; ++q) {
+    const double L = c[q], R = c[n + N - q];
+    std::vector<double> eta(n + 2, 0.0);   // eta_nu at nu + 1
+    double dp = 0.0;
+    for (int i = 0; i <= N; ++i) {
+      const double phi = i == q ? 1.0 : 0.0;
+      const double r = i == 0 ? 3.0 * phi + h * L : (i == N ? 3.0 * phi - h * R : 6.0 * phi);
+      dp = (r - dp) * lu[n + i];   // the first row has nothing before it: dp = 0
+      eta[i + 1] = dp;
+    }
+    for (int i = N - 1; i >= 0; --i) eta[i + 1] -= lu[i] * eta[i + 2];
+    eta[0] = eta[2] - 2.0 * h * L;
+    eta[N + 2] = eta[N] + 2.0 * h * R;
+    for (int k = 0; k < nk; ++k)
+      for (int j = 0; j < n; ++j) {
+        double acc = 0.0;
+        for (int t = 0; t < 4; ++t) {
+          const int nu = j - ns[k] - 2 + t;
+          if (nu >= -1 && nu <= N + 1) acc += w[4 * k + t] * eta[nu + 1];
+        }
+        out[((size_t)j * n + q) * nk + k] = acc;
+      }
+  }
+}
+
 int ensure_advect_tables(Handle* H, double tau) {
   if (H->adv.valid && H->adv.tau == tau) return CHASM_OK;
   const int nk = H->g.nk;
@@ -350,7 +382,7 @@ int ensure_advect_tables(Handle* H, double tau) {
     H->adv.ns_max[d] = *std::max_element(ns.begin() + (size_t)d * nk, ns.begin() + (size_t)(d + 1) * nk);
   }
   const size_t wbytes = w.size() * H->elt;
-  std::vector<unsigned char> blob(wbytes + ns.size() * sizeof(int));
+  std::vector<unsigned char> blob(advect_dense_offset(*H, 3));
   if (H->fp64)
     std::memcpy(blob.data(), w.data(), wbytes);
   else {
@@ -359,6 +391,10 @@ int ensure_advect_tables(Handle* H, double tau) {
     std::memcpy(blob.data(), wf.data(), wbytes);
   }
   std::memcpy(blob.data() + wbytes, ns.data(), ns.size() * sizeof(int));
+  for (int d = 0; d < 3; ++d)
+    if (advect_dense(*H, d))
+      dense_rows(H, d, &w[(size_t)d * nk * 4], &ns[(size_t)d * nk],
+                 reinterpret_cast<double*>(blob.data() + advect_dense_offset(*H, d)));
   int rc = upload(H, &H->adv.dev, blob.data(), blob.size());
   if (rc) return rc;
   CHASM_CUDA(H, cudaStreamSynchronize(H->stream));
@@ -762,6 +798,9 @@ size_t chasm_workspace_bytes(const chasm_grid* grid, const chasm_potential* pot,
   w += diag_bytes(grid->nx, nk);
   w += (size_t)3 * (grid->nx[0] + grid->nx[1] + grid->nx[2]) * (8 + 2 * e);
   w += (size_t)(grid->nx[0] + grid->nx[1] + grid->nx[2]) * nk * (fp64 ? 24 : 4) + 3 * nk * (4 * e + 4) + 16 * nk;
+  if (fp64)
+    for (int d = 0; d < 3; ++d)
+      if (grid->nx[d] <= kAdvDenseMax) w += (size_t)grid->nx[d] * grid->nx[d] * nk * 8;
   return w;
 }
 

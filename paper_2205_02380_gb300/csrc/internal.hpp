@@ -223,6 +223,19 @@ struct Handle {
   size_t workspace = 0;
 };
 
+// FP64 lines of up to kAdvDenseMax points in one patch are advected by dense matrices
+// (k_advect.cu): doubles [n * n][nk] per dimension behind the weights and shifts in AdvectTables::dev
+constexpr int kAdvDenseMax = 8;
+inline bool advect_dense(const Handle& H, int d) {
+  return H.fp64 && H.g.nx[d] <= kAdvDenseMax && H.opt.patches[d] <= 1;
+}
+inline size_t advect_dense_offset(const Handle& H, int dim) {   // dim = 3: the size of the whole table
+  size_t o = ((size_t)3 * H.g.nk * (4 * H.elt + sizeof(int)) + 15) / 16 * 16;
+  for (int d = 0; d < dim; ++d)
+    if (advect_dense(H, d)) o += (size_t)H.g.nx[d] * H.g.nx[d] * H.g.nk * sizeof(double);
+  return o;
+}
+
 // Returns a message for the last error on this thread when no handle exists.
 void set_thread_error(const std::string& e);
 

@@ -420,6 +420,32 @@ __global__ void __launch_bounds__(kAdvectThreads) k_advect_smem(AdvParams<T> p) 
   }
 }
 
+// ---- very short FP64 lines: the whole pass as a dense matrix per k ----
+// Closure, solve and evaluation of an n-point line cost about 7 + 2 J/n FP64 FMAs per point on a pipe
+// of 1.7 per clock and SM, the n x n matrix that they amount to costs n: less up to kAdvDenseMax
+// points (5 points: 1.75 -> 0.83 ms a pass at 121 x 5^2 x 32^3; 8 points run at 1175 GB/s, 9 points in
+// shared memory at 940).  The matrices come from the host
+// (dense_rows), entry (j, q) of every k side by side, so a warp reads one value or consecutive ones.
+template <int NX>
+__global__ void __launch_bounds__(kAdvectThreads) k_advect_dense(AdvParams<double> p, const double* __restrict__ mat) {
+  const int64_t line = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (line >= p.n_lines) return;
+  double* src;
+  int kd;
+  line_setup(p, line, src, kd);
+  double v[NX];
+#pragma unroll
+  for (int j = 0; j < NX; ++j) v[j] = src[(int64_t)j * p.s_d];
+  const double* m = mat + kd;
+#pragma unroll
+  for (int j = 0; j < NX; ++j) {
+    double acc = 0.0;
+#pragma unroll
+    for (int q = 0; q < NX; ++q) acc = fma(__ldg(m + (j * NX + q) * p.nk), v[q], acc);
+    src[(int64_t)j * p.s_d] = acc;
+  }
+}
+
 // ---- patches (p > 1): Sec. 3.1.2 steps (1)-(5) and the interpolation with correction of
 // Sec. 3.1.3, one line per thread in shared memory (column layout) ----
 template <typename T>
@@ -648,6 +674,20 @@ cudaError_t launch_t(const Handle& H, void* f, int dim, cudaStream_t s) {
     if (Bp == 0) return cudaErrorInvalidValue;
     k_advect_patches<T><<<(unsigned)((p.n_lines + Bp - 1) / Bp), Bp, elems * Bp * sizeof(T), s>>>(p, q);
     return cudaGetLastError();
+  }
+  if constexpr (sizeof(T) == 8) {
+    if (advect_dense(H, dim)) {
+      const double* mat = reinterpret_cast<const double*>(static_cast<const char*>(H.adv.dev) + advect_dense_offset(H, dim));
+      const unsigned nb = (unsigned)((p.n_lines + B - 1) / B);
+      switch (p.n) {
+        case 4: k_advect_dense<4><<<nb, B, 0, s>>>(p, mat); break;
+        case 5: k_advect_dense<5><<<nb, B, 0, s>>>(p, mat); break;
+        case 6: k_advect_dense<6><<<nb, B, 0, s>>>(p, mat); break;
+        case 7: k_advect_dense<7><<<nb, B, 0, s>>>(p, mat); break;
+        default: k_advect_dense<8><<<nb, B, 0, s>>>(p, mat); break;
+      }
+      return cudaGetLastError();
+    }
   }
   if (reg_applies(H, f, dim)) {
     const int64_t lpt = sizeof(T) == 4 ? 2 : 1;   // kvol = nk^3 is even
