@@ -122,6 +122,17 @@ __device__ __forceinline__ void load_pair(const float* src, float (&a)[N], float
     b[4 * q + 3] = v.w;
   }
 }
+// a, b += c2 times the pair at src
+template <int N>
+__device__ __forceinline__ void add_pair(const float* src, float c2, float (&a)[N], float (&b)[N]) {
+  float a2[N], b2[N];
+  load_pair<N>(src, a2, b2);
+#pragma unroll
+  for (int n = 0; n < N; ++n) {
+    a[n] = fmaf(c2, a2[n], a[n]);
+    b[n] = fmaf(c2, b2[n], b[n]);
+  }
+}
 template <int N>
 __device__ __forceinline__ void store_pair(float* dst, const float (&a)[N], const float (&b)[N]) {
   float4* d4 = reinterpret_cast<float4*>(dst);
@@ -135,15 +146,22 @@ __device__ __forceinline__ void store_pair(float* dst, const float (&a)[N], cons
 // The line pairs of one warp in a k3 pass (N = 32): lane k1 owns the pair (k1, k2 = 2m, 2m + 1)
 // with m common to the warp, i.e. 2N contiguous floats at src_m + k1 N^2.  Read through the warp's
 // slab buffer so that every global access of the warp covers two whole pairs (512 contiguous
-// bytes) instead of one 16-byte piece of 32 pairs: the loads no longer depend on L1 to merge.
-template <int N>
-__device__ __forceinline__ void warp_load_pairs(const float* src_m, float* T, float (&a)[N], float (&b)[N]) {
+// bytes) instead of one 16-byte piece of 32 pairs: the loads no longer depend on L1 to merge.  X2 and
+// src2_m: src + c2 src2, added on the way (two trips through the buffer made the LPC1 corrector
+// 4.46 ms at 24^3 x 32^3, one trip makes it 4.14).
+template <int N, bool X2>
+__device__ __forceinline__ void warp_load_pairs(const float* src_m, const float* src2_m, float c2, float* T,
+                                                float (&a)[N], float (&b)[N]) {
   constexpr int Q = N / 2, RW = 2 * N + 4;   // quads per pair, buffer row (floats)
   const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
     const int t = 2 * q + (lane >> 4), e = lane & 15;
-    const float4 v = __ldcs(reinterpret_cast<const float4*>(src_m + (size_t)t * N * N) + e);
+    float4 v = __ldcs(reinterpret_cast<const float4*>(src_m + (size_t)t * N * N) + e);
+    if (X2 && src2_m) {
+      const float4 w = __ldcs(reinterpret_cast<const float4*>(src2_m + (size_t)t * N * N) + e);
+      v = make_float4(fmaf(c2, w.x, v.x), fmaf(c2, w.y, v.y), fmaf(c2, w.z, v.z), fmaf(c2, w.w, v.w));
+    }
     *reinterpret_cast<float4*>(T + t * RW + 4 * e) = v;
   }
   __syncwarp();
@@ -308,17 +326,12 @@ __global__ void __launch_bounds__(PkCfg<N>::NT, PkCfg<N>::MINB) k_theta_pk(const
     const size_t off = (size_t)xq * N3 + ((size_t)k1 * N + 2 * m) * N;
     const size_t offm = (size_t)xq * N3 + (size_t)2 * m * N;   // the warp's common part (N = 32)
     float a[N], b[N];
-    if constexpr (!GSM) warp_load_pairs<N>(p.in + offm, Vw, a, b);
-    else load_pair<N>(p.in + off, a, b);
-    if (X2 && p.in2) {   // u_0 = in + cin2 in2 (the LPC1 predictor)
-      float a2[N], b2[N];
-      if constexpr (!GSM) warp_load_pairs<N>(p.in2 + offm, Vw, a2, b2);
-      else load_pair<N>(p.in2 + off, a2, b2);
-#pragma unroll
-      for (int n = 0; n < N; ++n) {
-        a[n] = fmaf(p.cin2, a2[n], a[n]);
-        b[n] = fmaf(p.cin2, b2[n], b[n]);
-      }
+    // u_0 = in + cin2 in2 (in2: the LPC1 predictor)
+    if constexpr (!GSM) {
+      warp_load_pairs<N, X2>(p.in + offm, X2 && p.in2 ? p.in2 + offm : nullptr, p.cin2, Vw, a, b);
+    } else {
+      load_pair<N>(p.in + off, a, b);
+      if (X2 && p.in2) add_pair<N>(p.in2 + off, p.cin2, a, b);
     }
     k3_forward<N, GSM>(a, b, G + (size_t)m * N + k1, pol);
   };
@@ -374,17 +387,11 @@ __global__ void __launch_bounds__(PkCfg<N>::NT, PkCfg<N>::MINB) k_theta_pk(const
         fft_pk<N, true>(y);
         float a[N], b[N];   // Horner base of the two lines
         if (p.base) {
-          if constexpr (!GSM) warp_load_pairs<N>(p.base + offm, Vw, a, b);
-          else load_pair<N>(p.base + off, a, b);
-          if (X2 && p.base2) {
-            float a2[N], b2[N];
-            if constexpr (!GSM) warp_load_pairs<N>(p.base2 + offm, Vw, a2, b2);
-            else load_pair<N>(p.base2 + off, a2, b2);
-#pragma unroll
-            for (int n = 0; n < N; ++n) {
-              a[n] = fmaf(p.cbase2, a2[n], a[n]);
-              b[n] = fmaf(p.cbase2, b2[n], b[n]);
-            }
+          if constexpr (!GSM) {
+            warp_load_pairs<N, X2>(p.base + offm, X2 && p.base2 ? p.base2 + offm : nullptr, p.cbase2, Vw, a, b);
+          } else {
+            load_pair<N>(p.base + off, a, b);
+            if (X2 && p.base2) add_pair<N>(p.base2 + off, p.cbase2, a, b);
           }
         } else {
 #pragma unroll
