@@ -63,9 +63,9 @@ cudaError_t launch_advect_dim(const Handle& H, void* f, int dim, cudaStream_t s)
 cudaError_t launch_theta(const Handle& H, const void* in, const void* base, void* out,
                          const double* coef, cudaStream_t s);
 struct ThetaPlan {
-  int cluster = 0;          // CTAs per cluster of the distributed-shared-memory kernel, 0 = global
-  int blocks = 0;           // grid size (a multiple of cluster)
-  size_t scratch_bytes = 0; // global scratch of the fallback kernel
+  int cluster = 0;          // modulated form: 1 = spectrum in shared memory, 0 = in global scratch
+  int blocks = 0;           // grid size
+  size_t scratch_bytes = 0; // global scratch
 };
 void theta_plan(int nk, bool fp64, int64_t nxp, int num_sms, ThetaPlan* plan);
 // real form with the per-x symbol table (k_theta_xs.cu): u_0 = in + cin2 in2, u_{s+1} =
@@ -115,6 +115,12 @@ void theta_pk_plan(int nk, int64_t nxp, int num_sms, ThetaPlan* plan);
 cudaError_t launch_theta_pk(const Handle& H, const void* in, const void* base, void* out, int nst,
                             const double* coef, cudaStream_t s, const XsExtra& x);
 
+// Modulated form in FP32 with N_k = 32 (k_theta_pk.cu); T-hat in the layout [s3][xi1 / 4][xi2][xi1 % 4]
+// (that_packed)
+__host__ __device__ constexpr bool that_packed(bool fp64, int nk) { return !fp64 && nk == 32; }
+void theta_mod_plan(int64_t nxp, int num_sms, ThetaPlan* plan);
+cudaError_t launch_theta_mod(const Handle& H, const void* in, const void* base, void* out, const double* coef,
+                             cudaStream_t s);
 // Double precision (k_theta_fx.cu): block fixed-point arithmetic.  Its symbol table is the FP64
 // table of nxp x points converted in place by fx_symbol, followed by fx_symbol_extra_bytes of
 // column exponents.

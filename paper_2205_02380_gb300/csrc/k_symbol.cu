@@ -154,13 +154,16 @@ __global__ void k_th_pass(const double* __restrict__ in, double* __restrict__ ou
 
 template <typename T>
 __global__ void k_that_store(const double* __restrict__ TH, T* __restrict__ that, int N) {
-  // TH[xi1][xi2][xi3] natural order -> that[s3][s1][s2] parity-major, / (2N)^3
+  // TH[xi1][xi2][xi3] natural order -> that[s3][s1][s2] parity-major, / (2N)^3; packed kernel:
+  // [s3][xi1 / 4][xi2][xi1 % 4]
   const int L = 2 * N;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= L * L * L) return;
   const int x3 = t % L, x2 = (t / L) % L, x1 = t / (L * L);
   const int s1 = (x1 & 1) * N + x1 / 2, s2 = (x2 & 1) * N + x2 / 2, s3 = (x3 & 1) * N + x3 / 2;
-  that[((int64_t)s3 * L + s1) * L + s2] = (T)(TH[t] / ((double)L * L * L));
+  const int64_t o = that_packed(sizeof(T) == 8, N) ? (((int64_t)s3 * (L / 4) + x1 / 4) * L + x2) * 4 + (x1 & 3)
+                                                   : ((int64_t)s3 * L + s1) * L + s2;
+  that[o] = (T)(TH[t] / ((double)L * L * L));
 }
 
 inline unsigned nblk(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }

@@ -21,8 +21,6 @@
 //   Phase C  2N^2 jobs: inverse FFT along k3, demodulate, Im, scale, accumulate per parity.
 //   Phase D  out = base + acc_0 + acc_1 (coalesced).
 // T-hat is stored in parity-major order [s3][s1][s2] with the 1/(2N)^3 normalisation folded in.
-#include <cooperative_groups.h>
-
 #include <cstdlib>
 #include <cstring>
 
@@ -31,8 +29,6 @@
 
 namespace chasm {
 namespace {
-
-namespace cg = cooperative_groups;
 
 
 template <typename T>
@@ -152,31 +148,21 @@ __global__ void __launch_bounds__(NT, MINB) k_theta(const ThetaParams<T> p) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// Cluster variant: the padded spectrum of one x point lives in distributed shared memory.
-//
-// A cluster of C CTAs owns one x point at a time.  CTA rank c keeps the slabs
-// s in [c SPC, (c+1) SPC), SPC = 2N / C, each N x (N+1) complex (padded rows), in its own shared
-// memory.  Phase A jobs of CTA c cover k1 in [c N/C, (c+1) N/C) and store their k3-spectra
-// straight into the owning CTA's slab (DSMEM stores, coalesced along k2); Phase B works on the
-// local slabs only; Phase C jobs read their k3-spectra back from the owners (DSMEM loads), do the
-// inverse transform, demodulate and write the output line.  Three cluster barriers per x point
-// and nucleus order the phases.  No global scratch is used.  For N <= 16 the whole spectrum fits
-// one CTA and C = 1.
+// Shared-memory variant (N <= 16): the padded spectrum of one x point, 2N slabs of N x (N+1) complex
+// (padded rows), stays in its CTA's shared memory; no global scratch is used.
 // ------------------------------------------------------------------------------------------------
-template <typename T, int N, int C>
+template <typename T, int N>
 struct ClCfg {
   static constexpr int NT = 256;
   static constexpr int L = 2 * N;
   static constexpr int GS = 2 * N;
   static constexpr int NG = NT / GS;
-  static constexpr int SPC = L / C;          // slabs per CTA
   static constexpr int SLAB = N * (N + 1);   // padded slab, complex entries
-  static constexpr int KPC = N / C;          // k1 rows per CTA in phases A and C
-  static_assert(NT % GS == 0 && N % C == 0 && (GS <= 32 || NG <= 15), "cluster tiling");
+  static_assert(NT % GS == 0 && (GS <= 32 || NG <= 15), "slab groups must tile the CTA");
   // slab buffers; the group buffers also hold the Phase C partials (NT x N reals)
   static constexpr size_t grp_cpx = (size_t)NG * N * VLayout<N>::VR;
   static constexpr size_t smem_cpx =
-      (size_t)SPC * SLAB + (grp_cpx * 2 >= (size_t)NT * N ? grp_cpx : ((size_t)NT * N + 1) / 2);
+      (size_t)L * SLAB + (grp_cpx * 2 >= (size_t)NT * N ? grp_cpx : ((size_t)NT * N + 1) / 2);
   static constexpr size_t smem_bytes = smem_cpx * sizeof(cpx<T>);
 };
 
@@ -194,42 +180,18 @@ struct ThetaClParams {
   T coef[kMaxNuclei];
 };
 
-template <int C>
-__device__ __forceinline__ void cluster_barrier() {
-  if constexpr (C == 1)
-    __syncthreads();
-  else
-    cg::this_cluster().sync();
-}
-
-template <typename T, int N, int C, int MINB>
+template <typename T, int N, int MINB>
 __global__ void __launch_bounds__(256, MINB) k_theta_cl(const ThetaClParams<T> p) {
-  using K = ClCfg<T, N, C>;
-  constexpr int L = K::L, GS = K::GS, NG = K::NG, NT = K::NT;
-  constexpr int SPC = K::SPC, SLAB = K::SLAB, KPC = K::KPC;
-  (void)NG;
+  using K = ClCfg<T, N>;
+  constexpr int L = K::L, GS = K::GS, NG = K::NG, NT = K::NT, SLAB = K::SLAB;
   constexpr int N3 = N * N * N;
   extern __shared__ __align__(16) unsigned char sm_raw[];
   cpx<T>* Gl = reinterpret_cast<cpx<T>*>(sm_raw);
   const int tid = threadIdx.x;
   const int grp = tid / GS, tg = tid % GS;
-  cpx<T>* V = Gl + SPC * SLAB + grp * (N * VLayout<N>::VR);
-  int rank = 0;
-  cpx<T>* Gr[C];
-  if constexpr (C == 1) {
-    Gr[0] = Gl;
-  } else {
-    cg::cluster_group cl = cg::this_cluster();
-    // launched without the matching cluster shape: touch no remote memory (uniform exit)
-    if (cl.num_blocks() != (unsigned)C || gridDim.x % C != 0) return;
-    rank = (int)cl.block_rank();
-#pragma unroll
-    for (int o = 0; o < C; ++o) Gr[o] = cl.map_shared_rank(Gl, o);
-    cl.sync();   // every CTA of the cluster is running before any remote shared-memory access
-  }
-  const int64_t cl_id = blockIdx.x / C, ncl = gridDim.x / C;
+  cpx<T>* V = Gl + L * SLAB + grp * (N * VLayout<N>::VR);
 
-  for (int64_t xp = cl_id; xp < p.nxp; xp += ncl) {
+  for (int64_t xp = blockIdx.x; xp < p.nxp; xp += gridDim.x) {
     const int i3 = (int)(xp % p.nx3);
     const int i2 = (int)((xp / p.nx3) % p.nx2);
     const int i1 = (int)(xp / ((int64_t)p.nx3 * p.nx2));
@@ -243,11 +205,11 @@ __global__ void __launch_bounds__(256, MINB) k_theta_cl(const ThetaClParams<T> p
       for (int q = 1; q < kMaxNuclei; ++q)
         if (q == a) coef = p.coef[q];
 
-      // ---- Phase A: modulate + twist + FFT along k3, scattered to the owners' slabs ----
+      // ---- Phase A: modulate + twist + FFT along k3, into the slabs ----
 #pragma unroll
       for (int r3 = 0; r3 < 2; ++r3) {
-        for (int job = tid; job < KPC * N; job += NT) {
-          const int k1 = rank * KPC + job / N, k2 = job % N;
+        for (int job = tid; job < N * N; job += NT) {
+          const int k1 = job / N, k2 = job % N;
           const int line = k1 * N + k2;
           const cpx<T> e12 = conjg(cmul(E1[k1], E2[k2]));
           T re[N], im[N];
@@ -261,33 +223,31 @@ __global__ void __launch_bounds__(256, MINB) k_theta_cl(const ThetaClParams<T> p
           fft<T, N, false>(re, im);
 #pragma unroll
           for (int j = 0; j < N; ++j) {
-            const int sg = r3 * N + j;        // global slab index (compile-time per j, r3)
-            Gr[sg / SPC][(sg % SPC) * SLAB + k1 * (N + 1) + k2] = {re[j], im[j]};
+            const int sg = r3 * N + j;        // slab index (compile-time per j, r3)
+            Gl[sg * SLAB + k1 * (N + 1) + k2] = {re[j], im[j]};
           }
         }
       }
-      cluster_barrier<C>();
+      __syncthreads();
 
-      // ---- Phase B: the local slabs, 2-D padded convolution in (k1, k2) ----
-      for (int sl = grp; sl < SPC; sl += NG) {
-        const int sg = rank * SPC + sl;
-        slab_conv<T, N, GS, N + 1, false>(Gl + sl * SLAB, V, p.that + (size_t)sg * L * L, tg, grp, 0);
-      }
-      cluster_barrier<C>();
+      // ---- Phase B: the slabs, 2-D padded convolution in (k1, k2) ----
+      for (int sl = grp; sl < L; sl += NG)
+        slab_conv<T, N, GS, N + 1, false>(Gl + sl * SLAB, V, p.that + (size_t)sl * L * L, tg, grp, 0);
+      __syncthreads();
 
       // ---- Phase C: inverse along k3 (both parities), demodulate, Im, write the line ----
-      for (int job = tid; job < KPC * N; job += NT) {
-        const int k1 = rank * KPC + job / N, k2 = job % N;
+      for (int job = tid; job < N * N; job += NT) {
+        const int k1 = job / N, k2 = job % N;
         const int line = k1 * N + k2;
         const cpx<T> e12 = cmul(E1[k1], E2[k2]);
-        T* P = reinterpret_cast<T*>(Gl + SPC * SLAB);   // parity-0 partials (idle group buffers)
+        T* P = reinterpret_cast<T*>(Gl + L * SLAB);   // parity-0 partials (idle group buffers)
         T re[N], im[N];
 #pragma unroll
         for (int r3 = 0; r3 < 2; ++r3) {
 #pragma unroll
           for (int j = 0; j < N; ++j) {
             const int sg = r3 * N + j;
-            const cpx<T> v = Gr[sg / SPC][(sg % SPC) * SLAB + k1 * (N + 1) + k2];
+            const cpx<T> v = Gl[sg * SLAB + k1 * (N + 1) + k2];
             re[j] = v.re;
             im[j] = v.im;
           }
@@ -307,7 +267,7 @@ __global__ void __launch_bounds__(256, MINB) k_theta_cl(const ThetaClParams<T> p
                                 : (p.base ? p.base + xp * N3 + (size_t)line * N : nullptr),
                           coef, re);
       }
-      cluster_barrier<C>();
+      __syncthreads();
     }
   }
 }
@@ -315,33 +275,24 @@ __global__ void __launch_bounds__(256, MINB) k_theta_cl(const ThetaClParams<T> p
 // ------------------------------------------------------------------------------------------------
 // Launch plans
 // ------------------------------------------------------------------------------------------------
-// global-scratch kernel configuration: one 512-thread CTA per SM for FP32 at N = 32 (the
-// per-CTA scratch then totals 152 x 512 KB, L2-resident); 256 threads otherwise
+// global-scratch kernel configuration: 256-thread CTAs, two per SM in FP32 (N <= 16)
 template <typename T, int N>
 constexpr int gs_threads() {
-  return (sizeof(T) == 4 && N == 32) ? 512 : 256;
+  return 256;
 }
 template <typename T, int N>
 constexpr int minb() {
-  return (sizeof(T) == 4 && N < 32) ? 2 : 1;
+  return sizeof(T) == 4 ? 2 : 1;
 }
 template <typename T, int N>
 size_t smem_bytes() {
   return (size_t)ThetaCfg<N, gs_threads<T, N>()>::smem_cpx * sizeof(cpx<T>);
 }
 
-// CTAs per SM the cluster kernel is compiled for (registers capped at 128 when 2)
+// CTAs per SM the shared-memory kernel is compiled for (registers capped at 128 when 2)
 template <typename T, int N>
 constexpr int cl_minb() {
-  return (sizeof(T) == 4 && N <= 16) ? 2 : 1;
-}
-
-// cluster size used for (T, N), 0 = global-scratch kernel
-template <typename T, int N>
-constexpr int cluster_size() {
-  if constexpr (N <= 16) return 1;
-  if constexpr (sizeof(T) == 4) return 4;
-  return 0;
+  return sizeof(T) == 4 ? 2 : 1;
 }
 
 template <typename T, int N>
@@ -357,52 +308,33 @@ int gs_occupancy() {
   return nb > 0 ? nb : 1;
 }
 
-template <typename T, int N, int C>
-int cl_max_clusters(int num_sms) {
-  using K = ClCfg<T, N, C>;
-  auto kern = k_theta_cl<T, N, C, cl_minb<T, N>()>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)K::smem_bytes) !=
-      cudaSuccess)
+// CTAs of the shared-memory kernel that run at once, 0 when it cannot
+template <typename T, int N>
+int cl_max_ctas(int num_sms) {
+  using K = ClCfg<T, N>;
+  auto kern = k_theta_cl<T, N, cl_minb<T, N>()>;
+  int nb = 0;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)K::smem_bytes) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, 256, K::smem_bytes) != cudaSuccess)
     return 0;
-  if constexpr (C == 1) {
-    int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, 256, K::smem_bytes) != cudaSuccess)
-      return 0;
-    return nb * num_sms;
-  } else {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(C * num_sms, 1, 1);
-    cfg.blockDim = dim3(256, 1, 1);
-    cfg.dynamicSmemBytes = K::smem_bytes;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = C;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) return 0;
-    return n;
-  }
+  return nb * num_sms;
 }
 
-// CHASM_THETA_VARIANT=global|cluster overrides the choice (both are parity-tested).
+// CHASM_THETA_VARIANT=global keeps the spectrum in global scratch for N <= 16 too (both are
+// parity-tested).
 template <typename T, int N>
 void plan_tn(int64_t nxp, int num_sms, ThetaPlan* pl) {
-  constexpr int C = cluster_size<T, N>();
   const char* env = std::getenv("CHASM_THETA_VARIANT");
-  const bool want_global = env ? std::strcmp(env, "global") == 0 : (C > 1);
-  if constexpr (C > 0) {
-   if (!want_global) {
-    const int ncl = cl_max_clusters<T, N, C>(num_sms);
-    if (ncl > 0) {
-      pl->cluster = C;
-      pl->blocks = (int)std::min<int64_t>(nxp, ncl) * C;
-      pl->scratch_bytes = 0;
-      return;
+  if constexpr (N <= 16) {
+    if (!(env && std::strcmp(env, "global") == 0)) {
+      const int n = cl_max_ctas<T, N>(num_sms);
+      if (n > 0) {
+        pl->cluster = 1;
+        pl->blocks = (int)std::min<int64_t>(nxp, n);
+        pl->scratch_bytes = 0;
+        return;
+      }
     }
-   }
   }
   pl->cluster = 0;
   pl->blocks = (int)std::min<int64_t>(nxp, (int64_t)gs_occupancy<T, N>() * num_sms);
@@ -413,9 +345,8 @@ template <typename T, int N>
 cudaError_t launch_tn(const Handle& H, const void* in, const void* base, void* out,
                       const double* coef, cudaStream_t s) {
   const int n_nuc = (int)H.nuclei.size();
-  if constexpr (cluster_size<T, N>() > 0) {
+  if constexpr (N <= 16) {
    if (H.theta.cluster > 0) {
-    constexpr int C = cluster_size<T, N>();
     ThetaClParams<T> p;
     p.in = static_cast<const T*>(in);
     p.base = static_cast<const T*>(base);
@@ -429,24 +360,8 @@ cudaError_t launch_tn(const Handle& H, const void* in, const void* base, void* o
     p.ph_stride = (int64_t)(H.g.nx[0] + H.g.nx[1] + 4 * H.g.nx[2]) * N;
     p.n_nuc = n_nuc;
     for (int a = 0; a < kMaxNuclei; ++a) p.coef[a] = a < n_nuc ? (T)coef[a] : (T)0;
-    if constexpr (C == 1) {
-      k_theta_cl<T, N, C, cl_minb<T, N>()><<<H.theta.blocks, 256, ClCfg<T, N, C>::smem_bytes, s>>>(p);
-      return cudaGetLastError();
-    } else {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)H.theta.blocks, 1, 1);
-      cfg.blockDim = dim3(256, 1, 1);
-      cfg.dynamicSmemBytes = ClCfg<T, N, C>::smem_bytes;
-      cfg.stream = s;
-      cudaLaunchAttribute attr;
-      attr.id = cudaLaunchAttributeClusterDimension;
-      attr.val.clusterDim.x = C;
-      attr.val.clusterDim.y = 1;
-      attr.val.clusterDim.z = 1;
-      cfg.attrs = &attr;
-      cfg.numAttrs = 1;
-      return cudaLaunchKernelEx(&cfg, k_theta_cl<T, N, C, cl_minb<T, N>()>, p);
-    }
+    k_theta_cl<T, N, cl_minb<T, N>()><<<H.theta.blocks, 256, ClCfg<T, N>::smem_bytes, s>>>(p);
+    return cudaGetLastError();
    }
   }
   ThetaParams<T> p;
@@ -480,7 +395,7 @@ cudaError_t launch_theta(const Handle& H, const void* in, const void* base, void
                     : launch_tn<float, 16>(H, in, base, out, coef, s);
     case 32:
       return H.fp64 ? launch_tn<double, 32>(H, in, base, out, coef, s)
-                    : launch_tn<float, 32>(H, in, base, out, coef, s);
+                    : launch_theta_mod(H, in, base, out, coef, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -494,7 +409,7 @@ void theta_plan(int nk, bool fp64, int64_t nxp, int num_sms, ThetaPlan* pl) {
       fp64 ? plan_tn<double, 16>(nxp, num_sms, pl) : plan_tn<float, 16>(nxp, num_sms, pl);
       return;
     case 32:
-      fp64 ? plan_tn<double, 32>(nxp, num_sms, pl) : plan_tn<float, 32>(nxp, num_sms, pl);
+      fp64 ? plan_tn<double, 32>(nxp, num_sms, pl) : theta_mod_plan(nxp, num_sms, pl);
       return;
   }
   pl->cluster = 0;

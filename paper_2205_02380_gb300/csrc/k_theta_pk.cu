@@ -419,6 +419,142 @@ __global__ void __launch_bounds__(PkCfg<N>::NT, PkCfg<N>::MINB) k_theta_pk(const
   }
 }
 
+// ---- modulated form (Eq. 4.6 per nucleus), N_k = 32 ----
+// The same packing for the complex convolution: per nucleus the lines are modulated by e^{-2i(x-x_A).k},
+// padded twofold along k3 as well, so the spectrum has 2N slabs (s3 = parity N + j), and every slab
+// is multiplied by T-hat.  A warp's lanes hold two neighbouring lines each, one parity at a time (the
+// modulation tables carry the odd parity's twist), and the slab phase is the one above; T-hat, 1 MB
+// and the same for every x point, stays in L2.  Before, a padded transform was split over two
+// threads with scalar arithmetic and shuffles: 3.41 -> 2.19 ms at 16^3 x 32^3, one nucleus.
+struct ModParams {
+  const float* in;
+  const float* base;    // may be null: out = Theta[in]; may alias out
+  float* out;
+  int64_t nxp;
+  int nx1, nx2, nx3;
+  const float* that;    // [2N][L/4][L][4]
+  const float2* ph;     // per nucleus E1[nx1][N], E2[nx2][N], E3[nx3][4][N] (forward even, odd; inverse even, odd)
+  int64_t ph_stride;
+  int n_nuc;
+  float coef[kMaxNuclei];
+  float4* G;            // per CTA: 2N slabs of N x N/2 quads
+};
+
+// (re, im) of the product of two packed complex numbers, the second the same in both lanes
+__device__ __forceinline__ pc mul_pc(const pc& a, float2 b) {
+  return {fma2(a.im, f2(-b.y, -b.y), mul2(a.re, f2(b.x, b.x))), fma2(a.im, f2(b.x, b.x), mul2(a.re, f2(b.y, b.y)))};
+}
+
+template <int N>
+__global__ void __launch_bounds__(PkCfg<N>::NT, 1) k_theta_mod(const ModParams p) {
+  using C = PkCfg<N>;
+  static_assert(!C::GSM, "N = 32");
+  constexpr int NT = C::NT, NW = C::NW, L = C::L, RS = C::RS;
+  constexpr int N3 = N * N * N, NP = N * N / 2, SQ = N * N / 2;
+  extern __shared__ __align__(16) float smf[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  float* Vw = smf + warp * C::VW;
+  float4* G = p.G + (size_t)blockIdx.x * 2 * C::GQ;
+  const uint64_t pol = l2_keep_policy();
+  for (int64_t xp = blockIdx.x; xp < p.nxp; xp += gridDim.x) {
+    const int i3 = (int)(xp % p.nx3), i2 = (int)((xp / p.nx3) % p.nx2), i1 = (int)(xp / ((int64_t)p.nx3 * p.nx2));
+    for (int nuc = 0; nuc < p.n_nuc; ++nuc) {
+      const float2* E1 = p.ph + nuc * p.ph_stride + (int64_t)i1 * N;
+      const float2* E2 = p.ph + nuc * p.ph_stride + (int64_t)(p.nx1 + i2) * N;
+      const float2* E3 = p.ph + nuc * p.ph_stride + (int64_t)(p.nx1 + p.nx2) * N + (int64_t)i3 * 4 * N;
+      float coef = p.coef[0];   // static indexing keeps the parameter block out of local memory
+#pragma unroll
+      for (int q = 1; q < kMaxNuclei; ++q)
+        if (q == nuc) coef = p.coef[q];
+      // e^{2i(x-x_A).k} of the pair's k1 and k2 (two lanes: k2 = 2m, 2m + 1)
+      auto e12 = [&](int k1, int m) {
+        const float2 u = __ldg(E1 + k1), a = __ldg(E2 + 2 * m), b = __ldg(E2 + 2 * m + 1);
+        return mul_pc(pc{f2(a.x, b.x), f2(a.y, b.y)}, u);
+      };
+
+      // ---- Phase A: modulate, k3 forward, both parities ----
+      for (int pr = tid; pr < NP; pr += NT) {
+        const int k1 = pr % N, m = pr / N;
+        float a[N], b[N];
+        warp_load_pairs<N, false>(p.in + (size_t)xp * N3 + (size_t)2 * m * N, nullptr, 0.f, Vw, a, b);
+        pc e = e12(k1, m);
+        e.im = f2(-e.im.x, -e.im.y);
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+          pc z[N];
+#pragma unroll
+          for (int n = 0; n < N; ++n) {
+            z[n] = mul_pc(e, __ldg(E3 + h * N + n));
+            z[n].re = mul2(z[n].re, f2(a[n], b[n]));
+            z[n].im = mul2(z[n].im, f2(a[n], b[n]));
+          }
+          fft_pk<N, false>(z);
+          float4* g = G + (size_t)h * N * SQ + (size_t)m * N + k1;
+#pragma unroll
+          for (int j = 0; j < N; ++j)
+            stg_keep4(g + (size_t)j * SQ, make_float4(z[j].re.x, z[j].re.y, z[j].im.x, z[j].im.y), pol);
+        }
+      }
+      __syncthreads();
+
+      // ---- Phase B: one warp per slab ----
+      for (int s = warp; s < L; s += NW) {
+        float4* gs = G + (size_t)s * SQ;
+        slab_rows_forward<N, false>(gs + lane, Vw + lane * RS, pol);
+        __syncwarp();
+#pragma unroll 1
+        for (int rnd = 0; rnd < 2; ++rnd)
+          slab_column<N>(Vw, lane + 32 * rnd, reinterpret_cast<const float4*>(p.that) + s * (int64_t)(L * L / 4), pol);
+        __syncwarp();
+        slab_rows_inverse<N, false>(gs + lane, Vw + lane * RS, pol);
+        __syncwarp();
+      }
+      __syncthreads();
+
+      // ---- Phase C: k3 inverse of both parities, demodulate, imaginary part ----
+      const float* base = nuc > 0 ? p.out : p.base;
+      for (int pr = tid; pr < NP; pr += NT) {
+        const int k1 = pr % N, m = pr / N;
+        const size_t offm = (size_t)xp * N3 + (size_t)2 * m * N;
+        const pc e = e12(k1, m);
+        float2 acc[N];
+#pragma unroll
+        for (int n = 0; n < N; ++n) acc[n] = f2(0.f, 0.f);
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+          const float4* g = G + (size_t)h * N * SQ + (size_t)m * N + k1;
+          pc y[N];
+#pragma unroll
+          for (int j = 0; j < N; ++j) {
+            const float4 v = ldg_keep4(g + (size_t)j * SQ, pol);
+            y[j] = {f2(v.x, v.y), f2(v.z, v.w)};
+          }
+          fft_pk<N, true>(y);
+#pragma unroll
+          for (int n = 0; n < N; ++n) {
+            const pc d = mul_pc(e, __ldg(E3 + (2 + h) * N + n));
+            acc[n] = fma2(d.re, y[n].im, fma2(d.im, y[n].re, acc[n]));
+          }
+        }
+        float a[N], b[N];
+        if (base) {
+          warp_load_pairs<N, false>(base + offm, nullptr, 0.f, Vw, a, b);
+        } else {
+#pragma unroll
+          for (int n = 0; n < N; ++n) a[n] = b[n] = 0.f;
+        }
+#pragma unroll
+        for (int n = 0; n < N; ++n) {
+          a[n] = fmaf(coef, acc[n].x, a[n]);
+          b[n] = fmaf(coef, acc[n].y, b[n]);
+        }
+        warp_store_pairs<N>(p.out + offm, Vw, a, b);
+      }
+      __syncthreads();   // G is reused by the next nucleus or x point
+    }
+  }
+}
+
 template <int N>
 void plan_pk_n(int64_t nxp, int num_sms, ThetaPlan* pl) {
   using C = PkCfg<N>;
@@ -467,6 +603,35 @@ cudaError_t launch_pk_n(const Handle& H, const void* in, const void* base, void*
 }
 
 }  // namespace
+
+void theta_mod_plan(int64_t nxp, int num_sms, ThetaPlan* pl) {
+  using C = PkCfg<32>;
+  cudaFuncSetAttribute(k_theta_mod<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_bytes);
+  pl->cluster = 0;
+  pl->blocks = (int)std::min<int64_t>(nxp, num_sms);
+  pl->scratch_bytes = (size_t)pl->blocks * 2 * C::GQ * sizeof(float4);
+}
+
+cudaError_t launch_theta_mod(const Handle& H, const void* in, const void* base, void* out, const double* coef,
+                             cudaStream_t s) {
+  using C = PkCfg<32>;
+  ModParams p;
+  p.in = static_cast<const float*>(in);
+  p.base = static_cast<const float*>(base);
+  p.out = static_cast<float*>(out);
+  p.nxp = H.g.nxp;
+  p.nx1 = H.g.nx[0];
+  p.nx2 = H.g.nx[1];
+  p.nx3 = H.g.nx[2];
+  p.that = static_cast<const float*>(H.d_that);
+  p.ph = static_cast<const float2*>(H.d_phase);
+  p.ph_stride = (int64_t)(H.g.nx[0] + H.g.nx[1] + 4 * H.g.nx[2]) * 32;
+  p.n_nuc = (int)H.nuclei.size();
+  for (int a = 0; a < kMaxNuclei; ++a) p.coef[a] = a < p.n_nuc ? (float)coef[a] : 0.f;
+  p.G = static_cast<float4*>(H.d_scratch);
+  k_theta_mod<32><<<H.theta.blocks, C::NT, C::smem_bytes, s>>>(p);
+  return cudaGetLastError();
+}
 
 bool theta_pk_applies(int nk, bool fp64) { return !fp64 && (nk == 16 || nk == 32); }
 
