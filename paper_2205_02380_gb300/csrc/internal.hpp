@@ -63,7 +63,7 @@ cudaError_t launch_advect_dim(const Handle& H, void* f, int dim, cudaStream_t s)
 cudaError_t launch_theta(const Handle& H, const void* in, const void* base, void* out,
                          const double* coef, cudaStream_t s);
 struct ThetaPlan {
-  int cluster = 0;          // modulated form: 1 = spectrum in shared memory, 0 = in global scratch
+  int cluster = 0;          // packed kernel: 2 = the last wave by pairs of CTAs; modulated form: 1 = spectrum in shared memory
   int blocks = 0;           // grid size
   size_t scratch_bytes = 0; // global scratch
 };

@@ -51,6 +51,7 @@ struct PkParams {
   int nst;             // stages, 1..4
   float ncoef[4];      // -c_s per stage (the sign of the deferred factor i); +c_s when REAL
   float4* G;           // per-CTA spectrum scratch [N][N/2][N] when it is not in shared memory
+  int64_t pair0;       // PAIRS: first x point done by two CTAs
 };
 
 template <int N>
@@ -303,22 +304,48 @@ __device__ __forceinline__ void slab_rows_inverse(float4* g, const float* vrow, 
   });
 }
 
+// Barrier of the CTAs that work on one x point: the CTA, or a cluster of two with the global spectrum
+// they exchange made visible.
+__device__ __forceinline__ void point_sync(bool two) {
+  if (two) {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  } else {
+    __syncthreads();
+  }
+}
+
+// The last wave (N = 32).  With PAIRS the CTAs come in clusters of two: x points up to p.pair0 are
+// done one per CTA as without it, the rest one per cluster, whose CTAs take slabs and line pairs
+// in turn and exchange the spectrum through the first one's scratch.  An x point takes 159 us of
+// P(dt) on one CTA and 98 on two, so a last wave of at most half the SMs is shorter by that
+// (plan_pk_n).
 // X2: the second input and base terms (in2, base2) are read (the LPC1 corrector).  REAL: the
 // table holds the real spectrum of an even kernel (the plain TKM convolution with T): no deferred
 // factor i, the result is Re[e^{i phi} y].
-template <int N, bool X2, bool REAL = false>
+template <int N, bool PAIRS, bool X2, bool REAL = false>
 __global__ void __launch_bounds__(PkCfg<N>::NT, PkCfg<N>::MINB) k_theta_pk(const PkParams p) {
   using C = PkCfg<N>;
-  constexpr int NT = C::NT, NW = C::NW, SPW = C::SPW, L = C::L, RS = C::RS;
+  constexpr int SPW = C::SPW, L = C::L, RS = C::RS;
   constexpr int N3 = N * N * N, NP = N * N / 2, SQ = N * N / 2;   // line pairs, quads per slab
   constexpr bool GSM = C::GSM;
+  static_assert(!PAIRS || !GSM, "a shared spectrum is in global scratch");
   extern __shared__ __align__(16) float smf[];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  float* Vw = smf + warp * C::VW;
-  float4* G = GSM ? reinterpret_cast<float4*>(smf + NW * C::VW) : p.G + (size_t)blockIdx.x * C::GQ;
+  const int lane = threadIdx.x & 31;
+  float* Vw = smf + (threadIdx.x >> 5) * C::VW;
   const uint64_t pol = l2_keep_policy();
   const uint64_t spol = l2_stream_policy();
   const int sub = lane / N, r = lane % N;
+  // the x points of this CTA, then (two) those of its cluster
+#pragma unroll 1
+  for (int two = 0; two < (PAIRS ? 2 : 1); ++two) {
+  const int64_t first = two ? p.pair0 + blockIdx.x / 2 : blockIdx.x, step = two ? gridDim.x / 2 : gridDim.x;
+  const int64_t end = PAIRS && !two ? p.pair0 : p.nxp;
+  // an x point's warps are numbered over its CTAs, neighbours on different ones
+  const int warp = two ? (int)(threadIdx.x >> 5) * 2 + (int)(blockIdx.x & 1) : (int)(threadIdx.x >> 5);
+  const int tid = warp * 32 + lane, NT = two ? 2 * C::NT : C::NT, NW = NT / 32;
+  float4* G = GSM ? reinterpret_cast<float4*>(smf + C::NW * C::VW) : p.G + (size_t)(two ? blockIdx.x & ~1u : blockIdx.x) * C::GQ;
+  if (PAIRS && two) point_sync(true);   // the other CTA is done with its own x points
 
   // Phase A for line pair pr of x point xq: k3 forward of the stage-0 input
   auto phase_a = [&](int64_t xq, int pr) {
@@ -335,19 +362,19 @@ __global__ void __launch_bounds__(PkCfg<N>::NT, PkCfg<N>::MINB) k_theta_pk(const
     }
     k3_forward<N, GSM>(a, b, G + (size_t)m * N + k1, pol);
   };
-  if (blockIdx.x < p.nxp) {
-    for (int pr = tid; pr < NP; pr += NT) phase_a(blockIdx.x, pr);
+  if (first < end) {
+    for (int pr = tid; pr < NP; pr += NT) phase_a(first, pr);
   }
-  __syncthreads();
+  point_sync(PAIRS && two);
 
-  for (int64_t xp = blockIdx.x; xp < p.nxp; xp += gridDim.x) {
+  for (int64_t xp = first; xp < end; xp += step) {
     for (int st = 0; st < p.nst; ++st) {
       // ---- Phase B: one warp per slab group ----
       for (int s0 = warp * SPW; s0 < N; s0 += NW * SPW) {
         if (lane == 0) {   // the symbol slabs this warp needs next, into L2
           const int sn = s0 + NW * SPW < N ? s0 + NW * SPW : warp * SPW;
-          const int64_t xn = s0 + NW * SPW < N || st + 1 < p.nst ? xp : xp + gridDim.x;
-          if (xn < p.nxp)
+          const int64_t xn = s0 + NW * SPW < N || st + 1 < p.nst ? xp : xp + step;
+          if (xn < end)
             bulk_prefetch_l2(p.sig + xn * p.sig_xs + sn * (int64_t)(L * L), SPW * L * L * sizeof(float));
         }
         float* Vs = Vw + sub * N * RS;
@@ -364,7 +391,7 @@ __global__ void __launch_bounds__(PkCfg<N>::NT, PkCfg<N>::MINB) k_theta_pk(const
         slab_rows_inverse<N, GSM>(gs + r, Vs + r * RS, pol);
         __syncwarp();
       }
-      __syncthreads();
+      point_sync(PAIRS && two);
 
       float nc = p.ncoef[0];   // static indexing keeps the parameter block out of local memory
 #pragma unroll
@@ -410,12 +437,13 @@ __global__ void __launch_bounds__(PkCfg<N>::NT, PkCfg<N>::MINB) k_theta_pk(const
           else store_pair<N>(p.out + off, a, b);
           // this thread alone used these spectrum columns: the next x point's Phase A for the
           // same line pair writes them without a barrier
-          if (xp + gridDim.x < p.nxp) phase_a(xp + gridDim.x, pr);
+          if (xp + step < end) phase_a(xp + step, pr);
         } else
           k3_forward<N, GSM>(a, b, g, pol);
       }
-      __syncthreads();
+      point_sync(PAIRS && two);
     }
+  }
   }
 }
 
@@ -555,21 +583,66 @@ __global__ void __launch_bounds__(PkCfg<N>::NT, 1) k_theta_mod(const ModParams p
   }
 }
 
+template <int N, bool PAIRS>
+void* pk_kernel(bool x2, bool real) {
+  if (real) return (void*)k_theta_pk<N, PAIRS, false, true>;
+  return x2 ? (void*)k_theta_pk<N, PAIRS, true> : (void*)k_theta_pk<N, PAIRS, false>;
+}
+template <int N, bool PAIRS>
+bool pk_set() {
+  bool ok = true;
+  for (int v = 0; v < 3; ++v)
+    ok &= cudaFuncSetAttribute(pk_kernel<N, PAIRS>(v == 1, v == 2), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)PkCfg<N>::smem_bytes) == cudaSuccess;
+  return ok;
+}
+// clusters of two CTAs that run at once
+template <int N>
+int pk_clusters(int num_sms) {
+  using C = PkCfg<N>;
+  if (!pk_set<N, true>()) return 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * (num_sms / 2));
+  cfg.blockDim = dim3(C::NT);
+  cfg.dynamicSmemBytes = C::smem_bytes;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim = {2, 1, 1};
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  return cudaOccupancyMaxActiveClusters(&n, pk_kernel<N, true>(false, false), &cfg) == cudaSuccess ? n : 0;
+}
+
+// One x point per CTA; with N_k = 32 the x points beyond the full waves are done by pairs of CTAs when
+// that is one wave of pairs and pairing loses no SM.  P(dt), 152 SMs, unpaired -> paired: 64 x points
+// 159 -> 98 us, 210 320 -> 267, 343 480 -> 430, 512 637 -> 595, 672 794 -> 757, 972 (6 full waves)
+// 1103 -> 1087; the CTAs drift apart over the waves, so that the pairs wait for their second half and
+// the gain is gone: 1584 (10 waves) 1722 -> 1742, 2197 (14) 2349 -> 2395.  Four CTAs per x point
+// were no faster than two.
+constexpr int kPairWaves = 6;
 template <int N>
 void plan_pk_n(int64_t nxp, int num_sms, ThetaPlan* pl) {
   using C = PkCfg<N>;
   int nb = 0;
-  cudaFuncSetAttribute(k_theta_pk<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_bytes);
-  cudaFuncSetAttribute(k_theta_pk<N, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)C::smem_bytes);
-  if (cudaFuncSetAttribute(k_theta_pk<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)C::smem_bytes) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_theta_pk<N, false>, C::NT, C::smem_bytes) !=
+  if (!pk_set<N, false>() ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, pk_kernel<N, false>(false, false), C::NT, C::smem_bytes) !=
           cudaSuccess ||
       nb < 1)
     nb = 1;
-  pl->cluster = 0;
-  pl->blocks = (int)std::min<int64_t>(nxp, (int64_t)nb * num_sms);
+  pl->cluster = 1;
+  const int64_t ctas = (int64_t)nb * num_sms;
+  pl->blocks = (int)std::min<int64_t>(nxp, ctas);
+  if constexpr (!C::GSM) {
+    const int64_t rest = nxp % ctas;
+    if (rest > 0 && nxp / ctas <= kPairWaves) {
+      const int64_t n = pk_clusters<N>(num_sms);
+      if (rest <= n && (nxp < ctas || 2 * n == ctas)) {
+        pl->cluster = 2;
+        pl->blocks = (int)(nxp < ctas ? 2 * rest : ctas);
+      }
+    }
+  }
   pl->scratch_bytes = C::GSM ? 0 : (size_t)pl->blocks * C::GQ * sizeof(float4);
 }
 
@@ -591,15 +664,25 @@ cudaError_t launch_pk_n(const Handle& H, const void* in, const void* base, void*
   p.nst = nst;
   for (int q = 0; q < 4; ++q) p.ncoef[q] = q < nst ? (float)(x.real_symbol ? coef[q] : -coef[q]) : 0.f;
   p.G = static_cast<float4*>(H.d_scratch);
-  if (x.real_symbol) {
-    if (x.in2 || x.base2) return cudaErrorInvalidValue;
-    k_theta_pk<N, false, true><<<H.theta.blocks, C::NT, C::smem_bytes, s>>>(p);
-  } else if (x.in2 || x.base2) {
-    k_theta_pk<N, true><<<H.theta.blocks, C::NT, C::smem_bytes, s>>>(p);
-  } else {
-    k_theta_pk<N, false><<<H.theta.blocks, C::NT, C::smem_bytes, s>>>(p);
+  const bool x2 = x.in2 || x.base2;
+  if (x.real_symbol && x2) return cudaErrorInvalidValue;
+  p.pair0 = H.g.nxp < H.theta.blocks ? 0 : H.g.nxp / H.theta.blocks * H.theta.blocks;
+  void* kern = pk_kernel<N, false>(x2, x.real_symbol);
+  if constexpr (!C::GSM) {
+    if (H.theta.cluster == 2) kern = pk_kernel<N, true>(x2, x.real_symbol);
   }
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)H.theta.blocks);
+  cfg.blockDim = dim3(C::NT);
+  cfg.dynamicSmemBytes = C::smem_bytes;
+  cfg.stream = s;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim = {2, 1, 1};
+  cfg.attrs = &attr;
+  cfg.numAttrs = H.theta.cluster > 1 ? 1 : 0;
+  void* args[] = {&p};
+  return cudaLaunchKernelExC(&cfg, kern, args);
 }
 
 }  // namespace
