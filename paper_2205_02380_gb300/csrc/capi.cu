@@ -598,7 +598,9 @@ int do_advect(Handle* H, void* f, double tau, bool tables_ready) {
     int rc = ensure_advect_tables(H, tau);
     if (rc) return rc;
   }
-  for (int d = 0; d < 3; ++d) CHASM_LAUNCH(H, launch_advect_dim(*H, f, d, H->stream));
+  if (advect_box(*H, f)) CHASM_LAUNCH(H, launch_advect_box(*H, f, H->stream));
+  else
+    for (int d = 0; d < 3; ++d) CHASM_LAUNCH(H, launch_advect_dim(*H, f, d, H->stream));
   return CHASM_OK;
 }
 

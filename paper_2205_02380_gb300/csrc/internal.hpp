@@ -59,6 +59,9 @@ inline int advect_smem_threads(size_t elems, size_t elt) {
 }
 cudaError_t advect_prepare();
 cudaError_t launch_advect_dim(const Handle& H, void* f, int dim, cudaStream_t s);
+// the three dimensions in one launch, where advect_box says that it applies
+bool advect_box(const Handle& H, const void* f);
+cudaError_t launch_advect_box(const Handle& H, void* f, cudaStream_t s);
 // Coulomb operator (k_theta.cu): out = (base or 0) + sum_a coef[a] * Theta_a[in]
 cudaError_t launch_theta(const Handle& H, const void* in, const void* base, void* out,
                          const double* coef, cudaStream_t s);

@@ -21,7 +21,8 @@
 // about 48 significant bits), i.e. at FP64-class precision without the FP64 pipe, which on GB300
 // delivers 1/64 of the FP32 rate and otherwise bounds this pass.  Everything else is FP32.
 //
-// Two kernels: k_advect_reg keeps the line in registers (integer shift in [-2, 1], the usual case
+// One kernel for the three dimensions of the smallest grids (k_advect_box), and per dimension:
+// k_advect_reg keeps the line in registers (integer shift in [-2, 1], the usual case
 // since |alpha| < 1; line length a compile-time constant from {16, 24, 32, 48, 64}, and in FP32
 // any length up to 64, in classes of four); k_advect_smem is the general fallback with the line
 // in shared memory (column layout, element e of thread t at e*B + t, conflict-free).
@@ -368,6 +369,95 @@ __global__ void __launch_bounds__(kAdvectThreads) k_advect_reg(AdvParams<T> p, c
       case 0: eval_line2<T, NX, 0>(v0, v1, wa, wb, st); break;
       default: eval_line2<T, NX, 1>(v0, v1, wa, wb, st); break;
     }
+  }
+}
+
+// ---- all three dimensions at once (FP32, the smallest grids) ----
+// A block holds the x grid of kBoxK consecutive k in shared memory and runs the three passes there: f
+// is read and written once, by one launch instead of three, whose latency bounds such a grid (what is
+// left is the chain of load, three solves and store: no ragged lengths, they would lengthen it).
+// Line lengths are compile-time constants; rows along x3 have an odd pitch, so that the lines of a
+// warp lie in different banks in every pass.
+constexpr int kBoxK = 4;
+constexpr int kBoxThreads = 256;
+constexpr int kBoxMaxNx = 16;
+constexpr int kBoxMaxNxp = 768;
+struct BoxArgs {
+  AdvParams<float> p[3];
+  AdvTabs<float> tb[3];
+};
+template <int NX>
+__device__ __forceinline__ void box_line(const AdvParams<float>& p, const AdvTabs<float>& tb, float* src, int sd,
+                                         int kd0, int kd1) {
+  constexpr int JC = NX;
+  float v0[NX + 2], v1[NX + 2];
+#pragma unroll
+  for (int j = 0; j < NX; ++j) {
+    const float2 q = *reinterpret_cast<const float2*>(src + j * sd);
+    v0[j + 1] = q.x;
+    v1[j + 1] = q.y;
+  }
+  solve_line<float, NX, JC>(p, tb, v0);
+  solve_line<float, NX, JC>(p, tb, v1);
+  const int sh0 = __ldg(p.ns + kd0), sh1 = __ldg(p.ns + kd1);
+  float wa[4], wb[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    wa[c] = __ldg(p.w + 4 * kd0 + c);
+    wb[c] = __ldg(p.w + 4 * kd1 + c);
+  }
+  auto eval = [&](int sh, auto&& st) {
+    switch (sh) {
+      case -2: eval_line2<float, NX, -2>(v0, v1, wa, wb, st); break;
+      case -1: eval_line2<float, NX, -1>(v0, v1, wa, wb, st); break;
+      case 0: eval_line2<float, NX, 0>(v0, v1, wa, wb, st); break;
+      default: eval_line2<float, NX, 1>(v0, v1, wa, wb, st); break;
+    }
+  };
+  // the two lines nearly always have one shift; where they straddle an integer, each its own
+  const int both = sh0 == sh1 ? 1 : 2;
+#pragma unroll 1
+  for (int q = 0; q < both; ++q)
+    eval(q ? sh1 : sh0, [&](int j, float a, float b) {
+      if (both == 1) *reinterpret_cast<float2*>(src + j * sd) = make_float2(a, b);
+      else src[j * sd + q] = q ? b : a;
+    });
+}
+__global__ void __launch_bounds__(kBoxThreads) k_advect_box(const __grid_constant__ BoxArgs a) {
+  extern __shared__ __align__(16) float box[];
+  const int n0 = a.p[0].n, n1 = a.p[1].n, n2 = a.p[2].n, P2 = n2 | 1;
+  const int64_t k0 = (int64_t)blockIdx.x * kBoxK;
+  float* f = a.p[0].f + k0;
+  const int64_t kvol = a.p[0].kvol;
+  constexpr int H = kBoxK / 2;   // pairs of k
+  const int nxp = n0 * n1 * n2;
+  for (int i = threadIdx.x; i < nxp * H; i += kBoxThreads) {
+    const int x = i / H, c = 2 * (i % H);
+    *reinterpret_cast<float2*>(box + (x / n2 * P2 + x % n2) * kBoxK + c) = *reinterpret_cast<const float2*>(f + x * kvol + c);
+  }
+#pragma unroll 1
+  for (int d = 0; d < 3; ++d) {
+    __syncthreads();
+    const AdvParams<float>& p = a.p[d];
+    const int lines = nxp / p.n;
+    const int sd = (d == 0 ? n1 * P2 : d == 1 ? P2 : 1) * kBoxK;
+    for (int i = threadIdx.x; i < lines * H; i += kBoxThreads) {
+      const int line = i / H, c = 2 * (i % H);
+      const int x = d == 2 ? line * P2 : line / n2 * (d == 0 ? P2 : n1 * P2) + line % n2;
+      float* src = box + x * kBoxK + c;
+      const int kd0 = (int)((k0 + c) / p.kdiv % p.nk), kd1 = (int)((k0 + c + 1) / p.kdiv % p.nk);
+      switch (p.n) {
+        case 4: box_line<4>(p, a.tb[d], src, sd, kd0, kd1); break;
+        case 8: box_line<8>(p, a.tb[d], src, sd, kd0, kd1); break;
+        case 12: box_line<12>(p, a.tb[d], src, sd, kd0, kd1); break;
+        default: box_line<16>(p, a.tb[d], src, sd, kd0, kd1); break;
+      }
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < nxp * H; i += kBoxThreads) {
+    const int x = i / H, c = 2 * (i % H);
+    *reinterpret_cast<float2*>(f + x * kvol + c) = *reinterpret_cast<const float2*>(box + (x / n2 * P2 + x % n2) * kBoxK + c);
   }
 }
 
@@ -729,6 +819,29 @@ cudaError_t advect_prepare() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_advect_patches<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAdvectMaxSmem);
   return e;
+}
+
+// The three passes in one launch, where a pass is bounded by its launch: N_k = 8 (128 blocks, fewer than
+// SMs; each has an x grid, so more k only add waves) and few x points.  FP32 Strang step, three
+// passes -> one: 4^3 27.8 -> 21.3 us, 8^3 33.4 -> 29.0, 12 x 8 x 8 41.2 -> 35.4, but 12^3 57.8 -> 60.0;
+// with N_k = 16 4^3 41.3 -> 49.7, 8^3 107.7 -> 118.7.
+bool advect_box(const Handle& H, const void* f) {
+  if (H.fp64 || H.g.nk != 8 || H.g.nxp > kBoxMaxNxp) return false;
+  for (int d = 0; d < 3; ++d)
+    if (!reg_applies(H, f, d) || H.g.nx[d] % 4 != 0 || H.g.nx[d] > kBoxMaxNx) return false;
+  return true;
+}
+
+cudaError_t launch_advect_box(const Handle& H, void* f, cudaStream_t s) {
+  BoxArgs a;
+  for (int d = 0; d < 3; ++d) {
+    a.p[d] = make_params<float>(H, f, d);
+    a.tb[d] = make_tabs<float>(H, d, false);
+  }
+  const size_t smem = (size_t)H.g.nx[0] * H.g.nx[1] * (H.g.nx[2] | 1) * kBoxK * sizeof(float);
+  static_assert(kBoxMaxNxp * 5 / 4 * kBoxK * sizeof(float) <= 48 * 1024, "without an opt-in");   // nx >= 4
+  k_advect_box<<<(unsigned)(H.g.kvol / kBoxK), kBoxThreads, smem, s>>>(a);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_advect_dim(const Handle& H, void* f, int dim, cudaStream_t s) {
