@@ -1,6 +1,6 @@
 // P-flow of the Coulomb operator in the real form, single precision, N_k = 16 and 32: the packed
-// (two-lane) variant of the table-form kernel (Sec. 4; the FP64 form and N_k = 8 run
-// k_theta_xs.cu).
+// (two-lane) variant of the table-form kernel (Sec. 4; N_k = 8 runs k_theta_xs.cu,
+// the FP64 form k_theta_fx.cu).
 //
 // It evaluates the same real linear convolution per x point,
 //   Theta^T[u]_p = sum_q S_{p-q}(x) u_q,  S_m(x) = sum_A c_A T_m sin(2 (x - x_A) . m dk),
