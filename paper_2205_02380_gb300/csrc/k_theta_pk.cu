@@ -318,34 +318,27 @@ __device__ __forceinline__ void point_sync(bool two) {
 // The last wave (N = 32).  With PAIRS the CTAs come in clusters of two: x points up to p.pair0 are
 // done one per CTA as without it, the rest one per cluster, whose CTAs take slabs and line pairs
 // in turn and exchange the spectrum through the first one's scratch.  An x point takes 159 us of
-// P(dt) on one CTA and 98 on two, so a last wave of at most half the SMs is shorter by that
-// (plan_pk_n).
-// X2: the second input and base terms (in2, base2) are read (the LPC1 corrector).  REAL: the
-// table holds the real spectrum of an even kernel (the plain TKM convolution with T): no deferred
-// factor i, the result is Re[e^{i phi} y].
-template <int N, bool PAIRS, bool X2, bool REAL = false>
-__global__ void __launch_bounds__(PkCfg<N>::NT, PkCfg<N>::MINB) k_theta_pk(const PkParams p) {
+// P(dt) on one CTA and 97 on two, so a last wave of at most half the SMs is shorter by that
+// (plan_pk_n).  The two kinds are separate copies of the code: with one for both, the kernel without
+// pairs was slower by 1.5 % (LPC1 corrector, 254 registers).
+// Every step-th x point from first to end, by one CTA or (TWO) by the two of a cluster, whose warps are
+// numbered so that neighbours are on different ones.
+template <int N, bool TWO, bool X2, bool REAL>
+__device__ __forceinline__ void pk_points(const PkParams& p, int64_t first, int64_t step, int64_t end) {
   using C = PkCfg<N>;
-  constexpr int SPW = C::SPW, L = C::L, RS = C::RS;
+  constexpr int NT = TWO ? 2 * C::NT : C::NT, NW = NT / 32, SPW = C::SPW, L = C::L, RS = C::RS;
   constexpr int N3 = N * N * N, NP = N * N / 2, SQ = N * N / 2;   // line pairs, quads per slab
   constexpr bool GSM = C::GSM;
-  static_assert(!PAIRS || !GSM, "a shared spectrum is in global scratch");
+  static_assert(!TWO || !GSM, "a shared spectrum is in global scratch");
   extern __shared__ __align__(16) float smf[];
   const int lane = threadIdx.x & 31;
+  const int warp = TWO ? (int)(threadIdx.x >> 5) * 2 + (int)(blockIdx.x & 1) : (int)(threadIdx.x >> 5);
+  const int tid = TWO ? warp * 32 + lane : threadIdx.x;
   float* Vw = smf + (threadIdx.x >> 5) * C::VW;
+  float4* G = GSM ? reinterpret_cast<float4*>(smf + C::NW * C::VW) : p.G + (size_t)(TWO ? blockIdx.x & ~1u : blockIdx.x) * C::GQ;
   const uint64_t pol = l2_keep_policy();
   const uint64_t spol = l2_stream_policy();
   const int sub = lane / N, r = lane % N;
-  // the x points of this CTA, then (two) those of its cluster
-#pragma unroll 1
-  for (int two = 0; two < (PAIRS ? 2 : 1); ++two) {
-  const int64_t first = two ? p.pair0 + blockIdx.x / 2 : blockIdx.x, step = two ? gridDim.x / 2 : gridDim.x;
-  const int64_t end = PAIRS && !two ? p.pair0 : p.nxp;
-  // an x point's warps are numbered over its CTAs, neighbours on different ones
-  const int warp = two ? (int)(threadIdx.x >> 5) * 2 + (int)(blockIdx.x & 1) : (int)(threadIdx.x >> 5);
-  const int tid = warp * 32 + lane, NT = two ? 2 * C::NT : C::NT, NW = NT / 32;
-  float4* G = GSM ? reinterpret_cast<float4*>(smf + C::NW * C::VW) : p.G + (size_t)(two ? blockIdx.x & ~1u : blockIdx.x) * C::GQ;
-  if (PAIRS && two) point_sync(true);   // the other CTA is done with its own x points
 
   // Phase A for line pair pr of x point xq: k3 forward of the stage-0 input
   auto phase_a = [&](int64_t xq, int pr) {
@@ -365,7 +358,7 @@ __global__ void __launch_bounds__(PkCfg<N>::NT, PkCfg<N>::MINB) k_theta_pk(const
   if (first < end) {
     for (int pr = tid; pr < NP; pr += NT) phase_a(first, pr);
   }
-  point_sync(PAIRS && two);
+  point_sync(TWO);
 
   for (int64_t xp = first; xp < end; xp += step) {
     for (int st = 0; st < p.nst; ++st) {
@@ -391,7 +384,7 @@ __global__ void __launch_bounds__(PkCfg<N>::NT, PkCfg<N>::MINB) k_theta_pk(const
         slab_rows_inverse<N, GSM>(gs + r, Vs + r * RS, pol);
         __syncwarp();
       }
-      point_sync(PAIRS && two);
+      point_sync(TWO);
 
       float nc = p.ncoef[0];   // static indexing keeps the parameter block out of local memory
 #pragma unroll
@@ -441,9 +434,22 @@ __global__ void __launch_bounds__(PkCfg<N>::NT, PkCfg<N>::MINB) k_theta_pk(const
         } else
           k3_forward<N, GSM>(a, b, g, pol);
       }
-      point_sync(PAIRS && two);
+      point_sync(TWO);
     }
   }
+}
+
+// X2: the second input and base terms (in2, base2) are read (the LPC1 corrector).  REAL: the
+// table holds the real spectrum of an even kernel (the plain TKM convolution with T): no deferred
+// factor i, the result is Re[e^{i phi} y].
+template <int N, bool PAIRS, bool X2, bool REAL = false>
+__global__ void __launch_bounds__(PkCfg<N>::NT, PkCfg<N>::MINB) k_theta_pk(const PkParams p) {
+  if constexpr (!PAIRS) {
+    pk_points<N, false, X2, REAL>(p, blockIdx.x, gridDim.x, p.nxp);
+  } else {
+    pk_points<N, false, X2, REAL>(p, blockIdx.x, gridDim.x, p.pair0);
+    point_sync(true);   // the other CTA is done with its own x points
+    pk_points<N, true, X2, REAL>(p, p.pair0 + blockIdx.x / 2, gridDim.x / 2, p.nxp);
   }
 }
 
@@ -616,10 +622,10 @@ int pk_clusters(int num_sms) {
 
 // One x point per CTA; with N_k = 32 the x points beyond the full waves are done by pairs of CTAs when
 // that is one wave of pairs and pairing loses no SM.  P(dt), 152 SMs, unpaired -> paired: 64 x points
-// 159 -> 98 us, 210 320 -> 267, 343 480 -> 430, 512 637 -> 595, 672 794 -> 757, 972 (6 full waves)
-// 1103 -> 1087; the CTAs drift apart over the waves, so that the pairs wait for their second half and
-// the gain is gone: 1584 (10 waves) 1722 -> 1742, 2197 (14) 2349 -> 2395.  Four CTAs per x point
-// were no faster than two.
+// 159 -> 97 us, 210 320 -> 267, 343 480 -> 424, 512 637 -> 580, 972 (6 full waves) 1103 -> 1046; the
+// CTAs drift apart over the waves, so that the pairs wait for their second half and the gain is
+// gone (one loop for both kinds of x points: 1584, 10 waves, 1722 -> 1742, 2197, 14 waves, 2349 ->
+// 2395).  Four CTAs per x point were no faster than two.
 constexpr int kPairWaves = 6;
 template <int N>
 void plan_pk_n(int64_t nxp, int num_sms, ThetaPlan* pl) {
