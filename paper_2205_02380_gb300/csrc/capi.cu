@@ -910,7 +910,8 @@ int chasm_create(const chasm_grid* grid, const chasm_box* box, const chasm_poten
         return bail(fail(H, CHASM_ENOMEM, "device allocation failed (Horner buffers / scratch)"));
     }
   }
-  if (H->nuclei.empty() && H->kappa != 0.0 && H->fp64) {
+  // chasm_theta needs kappa != 0, an LPC1 step applies Theta (then zero) without a potential too
+  if (H->nuclei.empty() && H->fp64 && (H->kappa != 0.0 || o.integrator == CHASM_LPC1)) {
     rc = build_kderiv(H);
     if (rc) return bail(rc);
   }

@@ -200,6 +200,7 @@ int64_t fx_spec_entry(double v) {
 }
 
 cudaError_t launch_kshift_fx(const Handle& H, void* f, int dim, const void* rows, const void* spec, cudaStream_t s) {
+  if (!rows || !spec) return cudaErrorInvalidValue;
   KPassParams p{};
   p.in = static_cast<const double*>(f);
   p.out = static_cast<double*>(f);
@@ -220,6 +221,7 @@ cudaError_t launch_kshift_fx(const Handle& H, void* f, int dim, const void* rows
 
 cudaError_t launch_kderiv_fx(const Handle& H, const void* in, const void* add, void* out, int dim, double coef,
                              cudaStream_t s) {
+  if (!H.d_kderiv) return cudaErrorInvalidValue;
   KPassParams p{};
   p.in = static_cast<const double*>(in);
   p.add = static_cast<const double*>(add);
