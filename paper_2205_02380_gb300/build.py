@@ -43,14 +43,16 @@ def _compile(src: str, verbose_ptxas: bool) -> str:
     return obj
 
 
+def dependencies() -> list:
+    """Every file the library is made from: all sources and headers, and this script."""
+    return ([os.path.join(CSRC, n) for n in sorted(os.listdir(CSRC)) if n.endswith((".cu", ".cuh", ".hpp"))]
+            + [os.path.join(HERE, "..", "include", "chasm.h"), os.path.abspath(__file__)])
+
+
 def build(verbose_ptxas: bool = False, force: bool = False) -> str:
     os.makedirs(BUILD, exist_ok=True)
-    srcs = [os.path.join(CSRC, s) for s in SOURCES]
-    deps = srcs + [os.path.join(CSRC, "internal.hpp"), os.path.join(CSRC, "fft_reg.cuh"),
-                   os.path.join(CSRC, "fft_pk.cuh"),
-                   os.path.join(HERE, "..", "include", "chasm.h")]
     if (not force and os.path.exists(LIB)
-            and os.path.getmtime(LIB) > max(os.path.getmtime(p) for p in deps)):
+            and os.path.getmtime(LIB) > max(os.path.getmtime(p) for p in dependencies())):
         return LIB
     with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
         objs = list(ex.map(lambda s: _compile(s, verbose_ptxas), SOURCES))
