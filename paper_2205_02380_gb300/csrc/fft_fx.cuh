@@ -74,9 +74,10 @@ __device__ __forceinline__ void xfor(F&& f) {
 }
 
 // ---- products ----
-// a b in 64 bits.  Written as its two halves: the compiler issues one wide product for them, and
-// four instructions for the C expression of the same product.
+// a b in 64 bits.  On the device written as its two halves: the compiler issues one wide product for
+// them, and four instructions for the C expression of the same product.
 __device__ __forceinline__ i64 fx_wide(int a, int b) {
+#ifdef __CUDA_ARCH__
   int hi;
   unsigned lo;
   i64 r;
@@ -84,20 +85,33 @@ __device__ __forceinline__ i64 fx_wide(int a, int b) {
   asm("mul.lo.s32 %0, %1, %2;" : "=r"(lo) : "r"(a), "r"(b));
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
   return r;
+#else
+  return (i64)a * (i64)b;
+#endif
+}
+// A constant w = C / 2^64 as 2^-32 (wh + wl / 2^32) with a signed low word.
+__host__ __device__ constexpr int fx_low(u64 c) { return (int)(unsigned)c; }
+__host__ __device__ constexpr unsigned fx_high(u64 c) { return (unsigned)((c >> 32) + (((unsigned)c) >> 31)); }
+// Whether the cross terms of x w, the high words of wh times the low word of x and of wl times its
+// signed high word, add up inside one signed word for every |x| < 2^62.7: below wh, and at most
+// |wl| 2^30.7 / 2^32 (2^30.7 < 0x67f80000) and one for its rounding.
+__host__ __device__ constexpr bool fx_one_word(u64 c) {
+  const i64 wl = fx_low(c);
+  const u64 cross = (u64)(wl < 0 ? -wl : wl) * 0x67f80000ULL >> 32;
+  return fx_high(c) + cross + 1 < (1ULL << 31);
 }
 // x w for a constant w = C / 2^64 < 1/2, rounded down to within two units; |x| < 2^62.7.  The
-// constant's low word is taken as signed, so both cross terms are single high products.  Their
-// sum fits one word for w < 1/3 (the first is below 2^32 / 3, the second below 2^29.7 in
-// magnitude).
+// constant's low word is taken as signed, so both cross terms are single high products; where the
+// constant allows it (fx_one_word) they are added in 32 bits.
 template <u64 C>
 __device__ __forceinline__ i64 fx_mulc(i64 x) {
   static_assert(C < (1ULL << 63) - (1ULL << 32), "constants below one half");
-  constexpr int wl = (int)(unsigned)C;
-  constexpr unsigned wh = (unsigned)((C >> 32) + (((unsigned)C) >> 31));
+  constexpr int wl = fx_low(C);
+  constexpr unsigned wh = fx_high(C);
   const int xh = (int)(x >> 32);
   const unsigned xl = (unsigned)x;
   const int b = __mulhi(wl, xh);
-  if constexpr (wh < 0x55555555u) {
+  if constexpr (fx_one_word(C)) {
     return fx_wide((int)wh, xh) + (i64)(int)(__umulhi(wh, xl) + (unsigned)b);
   } else {
     return fx_wide((int)wh, xh) + (i64)(u64)__umulhi(wh, xl) + (i64)b;
