@@ -46,7 +46,8 @@ enum {
   CHASM_EUNSTABLE = -4,   /* dt * rho(Theta^T) above the Taylor-4 stability limit 2.8          */
   CHASM_EBUSY = -5,       /* server: request larger than the whole HBM budget                  */
   CHASM_EAGAIN = -6,      /* server: submission queue full, retry later                        */
-  CHASM_ETIMEOUT = -7,    /* chasm_wait: timed out                                             */
+  CHASM_ETIMEOUT = -7,    /* chasm_wait: timed out; calls that wait for a handle's stream: a bounded
+                             wait inside a kernel ran out, what the kernel wrote is NaN        */
   CHASM_ENOTFOUND = -8,   /* server: unknown ticket                                            */
   CHASM_ECANCELED = -9    /* server: request cancelled before it finished                      */
 };
@@ -168,7 +169,8 @@ size_t chasm_f_bytes(const chasm_handle* h);
  * Drops captured graphs. */
 int chasm_set_stream(chasm_handle* h, void* cuda_stream);
 
-/* Waits for all work issued on the handle's stream; reports asynchronous CUDA errors. */
+/* Waits for all work issued on the handle's stream; reports asynchronous CUDA errors and, once,
+ * a wait inside a kernel that ran out (ETIMEOUT). */
 int chasm_sync(chasm_handle* h);
 
 /* nsteps steps of the handle's integrator (Strang: S(dt) = A(dt/2) P(dt) A(dt/2); LPC1: the

@@ -680,6 +680,16 @@ int issue_step_lpc1(Handle* H, void* f, double dt) {
   return theta_any(H, V, f, f, 0.5 * dt);
 }
 
+// The double-precision table-form kernel hands data between warps through barriers whose waits end; one that
+// ran out leaves NaN and sets the late word.  Read here by the calls that wait for the stream, after
+// `late` has been copied with their results, and cleared.
+bool has_late_word(const Handle* H) { return H->fp64 && H->xs; }
+int late_status(Handle* H, int late) {
+  if (!late) return CHASM_OK;
+  CHASM_CUDA(H, cudaMemsetAsync(late_word(*H), 0, sizeof(int), H->stream));
+  return fail(H, CHASM_ETIMEOUT, "a wait inside the double-precision Coulomb kernel ran out; its results are NaN");
+}
+
 int prepare_step(Handle* H, double dt) {
   if (!is_finite(dt) || !(dt > 0)) return fail(H, CHASM_EINVAL, "dt must be > 0 and finite");
   if (H->opt.integrator == CHASM_LPC1) {
@@ -880,6 +890,8 @@ int chasm_create(const chasm_grid* grid, const chasm_box* box, const chasm_poten
       cudaMallocAsync((void**)&H->d_result, sizeof(double) * 4, H->stream) != cudaSuccess ||
       cudaMallocAsync((void**)&H->d_diag, diag_bytes(g.nx, g.nk), H->stream) != cudaSuccess)
     return bail(fail(H, CHASM_ENOMEM, "device allocation failed (reductions)"));
+  e = cudaMemsetAsync(H->d_result, 0, sizeof(double) * 4, H->stream);   // the late word among them
+  if (e != cudaSuccess) return bail(cuda_fail(H, e, "reductions"));
   const size_t fbytes = (size_t)g.ncell * H->elt;
   if (!H->nuclei.empty()) {
     const int N = g.nk;
@@ -967,9 +979,12 @@ int chasm_launch_count(const chasm_handle* h, int64_t* out) {
 int chasm_sync(chasm_handle* h) {
   Handle* H = reinterpret_cast<Handle*>(h);
   if (!H) return fail(nullptr, CHASM_EINVAL, "handle is NULL");
+  int late = 0;
+  if (has_late_word(H))
+    CHASM_CUDA(H, cudaMemcpyAsync(&late, late_word(*H), sizeof(late), cudaMemcpyDeviceToHost, H->stream));
   CHASM_CUDA(H, cudaStreamSynchronize(H->stream));
   CHASM_CUDA(H, cudaGetLastError());
-  return CHASM_OK;
+  return late_status(H, late);
 }
 
 int chasm_step(chasm_handle* h, void* f, double dt, int32_t nsteps) {
@@ -1070,12 +1085,14 @@ int chasm_moments(chasm_handle* h, const void* f, double* mass, double* energy) 
   if (!H) return fail(nullptr, CHASM_EINVAL, "handle is NULL");
   if (!f) return fail(H, CHASM_EINVAL, "f is NULL");
   CHASM_CUDA(H, launch_moments(*H, f, H->d_partials, H->d_result, H->stream));
-  double r[2];
+  double r[3];   // mass, energy, the late word
   CHASM_CUDA(H, cudaMemcpyAsync(r, H->d_result, sizeof(r), cudaMemcpyDeviceToHost, H->stream));
   CHASM_CUDA(H, cudaStreamSynchronize(H->stream));
   if (mass) *mass = r[0];
   if (energy) *energy = r[1];
-  return CHASM_OK;
+  int late;
+  std::memcpy(&late, &r[2], sizeof(late));
+  return late_status(H, late);
 }
 
 namespace {
@@ -1086,8 +1103,7 @@ int diag_call(chasm_handle* h, const void* f, int what, int j, double* out, size
   double* res = H->d_diag + (size_t)3 * H->g.nxp * H->g.nk;
   CHASM_CUDA(H, launch_diag(*H, f, what, j, H->d_diag, res, H->stream));
   CHASM_CUDA(H, cudaMemcpyAsync(out, res, n * sizeof(double), cudaMemcpyDeviceToHost, H->stream));
-  CHASM_CUDA(H, cudaStreamSynchronize(H->stream));
-  return CHASM_OK;
+  return chasm_sync(h);
 }
 }  // namespace
 

@@ -232,6 +232,9 @@ struct Handle {
   size_t workspace = 0;
 };
 
+// the word behind the moments' two results that a kernel sets when a bounded wait in it ran out
+inline int* late_word(const Handle& H) { return reinterpret_cast<int*>(H.d_result + 2); }
+
 // FP64 lines of up to kAdvDenseMax points in one patch are advected by dense matrices
 // (k_advect.cu): doubles [n * n][nk] per dimension behind the weights and shifts in AdvectTables::dev
 constexpr int kAdvDenseMax = 8;

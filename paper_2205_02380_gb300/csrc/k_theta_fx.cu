@@ -43,6 +43,7 @@
 #include "internal.hpp"
 #include "fft_reg.cuh"
 #include "fft_fx.cuh"
+#include "group_bar.cuh"
 
 namespace chasm {
 namespace {
@@ -62,6 +63,7 @@ struct FxParams {
   int nst;             // stages, 1..4
   double coef[4];      // c_s per stage
   fxc* G;              // per-CTA spectrum scratch when it is not in shared memory
+  int* late;           // set when a wait ran out (chasm_sync reports it)
 };
 
 template <int N>
@@ -82,29 +84,6 @@ struct FxCfg {
   static constexpr size_t smem_bytes = v_bytes + g_bytes + e_bytes;
   static_assert(NG * VSZ * sizeof(fxc) / NW >= 32 * TROW * 16, "line staging fits the slab buffers");
 };
-
-// ---- barriers between the two warps of a group (mbarriers in shared memory) ----
-__device__ __forceinline__ unsigned sm_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mb_init(unsigned b, int warps) {
-  asm volatile("mbarrier.init.shared.b64 [%0], %1;" ::"r"(b), "r"(warps) : "memory");
-}
-// this warp's arrival: what its lanes did before is visible to whoever waits for the phase
-__device__ __forceinline__ void mb_arrive(unsigned b) {
-  __syncwarp();
-  if ((threadIdx.x & 31) == 0) asm volatile("mbarrier.arrive.shared.b64 _, [%0];" ::"r"(b) : "memory");
-  __syncwarp();
-}
-// waits for the end of a phase of this parity; false when it has not come after about a second
-__device__ __forceinline__ bool mb_wait(unsigned b, int parity) {
-  unsigned done = 0;
-  for (int i = 0; !done && i < (1 << 20); ++i)
-    asm volatile("{\n .reg .pred q;\n mbarrier.try_wait.parity.shared.b64 q, [%1], %2;\n selp.u32 %0, 1, 0, q;\n}"
-                 : "=r"(done)
-                 : "r"(b), "r"(parity & 1)
-                 : "memory");
-  __syncwarp();
-  return done != 0;
-}
 
 template <int N>
 __device__ __forceinline__ int seg_max(int v) {   // over the aligned groups of N lanes
@@ -297,6 +276,7 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
   using C = FxCfg<N>;
   constexpr int L = C::L, SPW = C::SPW, NG = C::NG, NW = C::NW, VR = C::VR, N2 = N * N, N3 = N * N * N;
   constexpr bool GSM = C::GSM;
+  constexpr bool FW = N == 8;   // P(dt) at 24^3 x 8^3 1.425 -> 1.410 ms, at 24^3 x 16^3 11.03 -> 11.34
   extern __shared__ __align__(16) unsigned char smem[];
   const FxShared<N> S(smem, p.G);
   const uint64_t pol = l2_keep_policy(), spol = l2_stream_policy();
@@ -324,7 +304,6 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
     auto off = [&](int t) { return (size_t)xp * N3 + ((size_t)(t % N) * N + item * SPW + t / N) * N; };
     fxc x[N];
     int E = 0, em = 1;
-    bool ok = true;
 #pragma unroll 1
     for (int step = first; step <= final; ++step) {
       const bool odd = !lines && (step < 3) == (S.wb == 1);   // this warp's half of the padded transform
@@ -406,7 +385,7 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
         }
         S.ex1[(S.sub * 2 + (odd ? 1 : 0)) * N + S.ln] = make_int2(E, E + mag_bits(m));
         mb_arrive(S.bar + kBoth);
-        ok &= mb_wait(S.bar + kBoth, 0);
+        mb_wait<FW>(S.bar + kBoth, 0, S.flag);
       } else if (step == kColF0 || step == kColF1) {
         const int64_t j = s0 + sc;
         const i64* sg = p.sig + xp * p.sig_xs + ((j * L + (odd ? N : 0)) * L + c);
@@ -427,13 +406,13 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
       } else if (step == kColB0 || step == kColB1) {
         fxc* col = S.V + (size_t)sc * N * VR + c;
         if (!odd) {
-          ok &= mb_wait(S.bar + kRead, turn);
+          mb_wait<FW>(S.bar + kRead, turn, S.flag);
 #pragma unroll
           for (int n = 0; n < N; ++n) col[n * VR] = x[n];
           S.exP[cc] = E;
           mb_arrive(S.bar + kWritten);
         } else {
-          ok &= mb_wait(S.bar + kWritten, turn);
+          mb_wait<FW>(S.bar + kWritten, turn, S.flag);
           const int ep = S.exP[cc], et = max(ep, E) + 1;
           const int s0_ = shift_of(et, ep), s1_ = shift_of(et, E);
           unsigned m = 0;
@@ -450,7 +429,7 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
         ++turn;
         if (step == kColB1) {
           mb_arrive(S.bar + kBoth);
-          ok &= mb_wait(S.bar + kBoth, 1);
+          mb_wait<FW>(S.bar + kBoth, 1, S.flag);
         }
       } else if (step == kRowB) {
         fxc* row = S.V + (S.sub * N + S.ln) * VR;
@@ -458,9 +437,9 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
 #pragma unroll
           for (int n = 0; n < N; ++n) row[n] = x[n];
           mb_arrive(S.bar + kWritten);
-          ok &= mb_wait(S.bar + kRead, turn);
+          mb_wait<FW>(S.bar + kRead, turn, S.flag);
         } else {
-          ok &= mb_wait(S.bar + kWritten, turn);
+          mb_wait<FW>(S.bar + kWritten, turn, S.flag);
           fxc* g = S.G + (size_t)(s0 + S.sub) * N2 + S.ln;
           unsigned m = 0;
 #pragma unroll
@@ -501,7 +480,6 @@ __device__ __forceinline__ void fx_phase(const FxParams& p, int64_t xp, int st, 
         S.exA[(item * SPW + S.sub) * N + S.ln] = make_int2(E, E + mag_bits(m));
       }
     }
-    if (!ok) *S.flag = 1;   // an exchange never came: no result rather than a wrong one
   }
 }
 
@@ -515,9 +493,12 @@ __global__ void __launch_bounds__(FxCfg<N>::NT, 1) k_theta_fx(const FxParams p) 
     mb_init(b + kWritten, 1);
     mb_init(b + kBoth, 2);
   }
+  // flag[0]: this x point becomes NaN; flag[1]: an exchange never came, no results from then on rather
+  // than wrong ones
+  if (threadIdx.x == 0) S.flag[1] = 0;
   int turn = 0;
   for (int64_t xp = blockIdx.x; xp < p.nxp; xp += gridDim.x) {
-    if (threadIdx.x == 0) *S.flag = 0;
+    if (threadIdx.x == 0) S.flag[0] = S.flag[1];
     __syncthreads();
 #pragma unroll 1
     for (int ph = 1; ph < 2 * p.nst + 2; ++ph) {   // lines of the input, then slabs and lines per stage
@@ -531,6 +512,7 @@ __global__ void __launch_bounds__(FxCfg<N>::NT, 1) k_theta_fx(const FxParams p) 
       }
     }
   }
+  if (threadIdx.x == 0 && S.flag[1]) *p.late = 1;
 }
 
 // sigma (FP64, [x][j][s1][s2]) -> fixed point in place: the N values of a column (one parity of
@@ -593,6 +575,7 @@ cudaError_t launch_fx_n(const Handle& H, const void* in, const void* base, void*
   p.nst = nst;
   for (int q = 0; q < 4; ++q) p.coef[q] = q < nst ? coef[q] : 0.0;
   p.G = static_cast<fxc*>(H.d_scratch);
+  p.late = late_word(H);
   if (x.real_symbol) {
     if (x.in2 || x.base2) return cudaErrorInvalidValue;
     k_theta_fx<N, false, true><<<H.theta.blocks, C::NT, C::smem_bytes, s>>>(p);
