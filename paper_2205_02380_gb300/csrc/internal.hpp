@@ -43,9 +43,10 @@ struct Handle;
 // advection (k_advect.cu)
 constexpr int kAdvectThreads = 128;
 constexpr int kAdvectMaxSmem = 200 * 1024;
-// shared-memory elements per line of the general advection kernel: the line (n + 2), and for
-// p > 1 patches the line, the p + 1 closure values (hi and lo parts) and the p (M + 3) patch
-// coefficients
+// Shared-memory elements per line of the general advection kernel: the line (n + 2).  For p > 1 patches
+// this is only the measure of the longest line that chasm_create accepts (a line, p + 1 closure values
+// in two parts and all patches' p (M + 3) coefficients); the patched kernel needs less and sizes its
+// launch itself.
 inline size_t advect_smem_elems(int n, int p) {
   return p > 1 ? (size_t)n + 2 * (p + 1) + (size_t)p * ((n - 1) / p + 3) : (size_t)n + 2;
 }
