@@ -46,8 +46,8 @@ enum {
   CHASM_EUNSTABLE = -4,   /* dt * rho(Theta^T) above the Taylor-4 stability limit 2.8          */
   CHASM_EBUSY = -5,       /* server: request larger than the whole HBM budget                  */
   CHASM_EAGAIN = -6,      /* server: submission queue full, retry later                        */
-  CHASM_ETIMEOUT = -7,    /* chasm_wait: timed out; calls that wait for a handle's stream: a bounded
-                             wait inside a kernel ran out, what the kernel wrote is NaN        */
+  CHASM_ETIMEOUT = -7,    /* chasm_wait: timed out; chasm_moments: a bounded wait inside a kernel ran
+                             out since the last call, what the kernel wrote is NaN             */
   CHASM_ENOTFOUND = -8,   /* server: unknown ticket                                            */
   CHASM_ECANCELED = -9    /* server: request cancelled before it finished                      */
 };
@@ -169,8 +169,7 @@ size_t chasm_f_bytes(const chasm_handle* h);
  * Drops captured graphs. */
 int chasm_set_stream(chasm_handle* h, void* cuda_stream);
 
-/* Waits for all work issued on the handle's stream; reports asynchronous CUDA errors and, once,
- * a wait inside a kernel that ran out (ETIMEOUT). */
+/* Waits for all work issued on the handle's stream; reports asynchronous CUDA errors. */
 int chasm_sync(chasm_handle* h);
 
 /* nsteps steps of the handle's integrator (Strang: S(dt) = A(dt/2) P(dt) A(dt/2); LPC1: the
@@ -207,7 +206,8 @@ int chasm_theta(chasm_handle* h, const void* u_dev, void* out_dev);
 int chasm_tkm_convolve(chasm_handle* h, const void* g_dev, void* phi_dev);
 
 /* Mass h1 h2 h3 dk^3 sum f and energy h1 h2 h3 dk^3 sum (hbar^2 |k|^2 / 2m + V(x)) f, both
- * accumulated in FP64 with a fixed reduction tree (bitwise reproducible); synchronous. */
+ * accumulated in FP64 with a fixed reduction tree (bitwise reproducible); synchronous.  ETIMEOUT, once:
+ * a wait inside a kernel of this handle ran out (CHASM_ETIMEOUT above). */
 int chasm_mass(chasm_handle* h, const void* f_dev, double* out);
 int chasm_energy(chasm_handle* h, const void* f_dev, double* out);
 int chasm_moments(chasm_handle* h, const void* f_dev, double* mass, double* energy);

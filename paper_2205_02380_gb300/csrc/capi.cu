@@ -542,7 +542,7 @@ int build_phase_tables(Handle* H) {
 
 int build_potential_table(Handle* H) {
   const int* nx = H->g.nx;
-  std::vector<double> v((size_t)H->g.nxp);
+  std::vector<double> v((size_t)H->g.nxp + 1);   // and the late word, zero
   size_t idx = 0;
   for (int i1 = 0; i1 < nx[0]; ++i1)
     for (int i2 = 0; i2 < nx[1]; ++i2)
@@ -681,9 +681,8 @@ int issue_step_lpc1(Handle* H, void* f, double dt) {
 }
 
 // The double-precision table-form kernel hands data between warps through barriers whose waits end; one that
-// ran out leaves NaN and sets the late word.  Read here by the calls that wait for the stream, after
-// `late` has been copied with their results, and cleared.
-bool has_late_word(const Handle* H) { return H->fp64 && H->xs; }
+// ran out leaves NaN and sets the late word, which chasm_moments reads with its results (a copy of its own in
+// chasm_sync took 8 us) and clears here.
 int late_status(Handle* H, int late) {
   if (!late) return CHASM_OK;
   CHASM_CUDA(H, cudaMemsetAsync(late_word(*H), 0, sizeof(int), H->stream));
@@ -890,8 +889,6 @@ int chasm_create(const chasm_grid* grid, const chasm_box* box, const chasm_poten
       cudaMallocAsync((void**)&H->d_result, sizeof(double) * 4, H->stream) != cudaSuccess ||
       cudaMallocAsync((void**)&H->d_diag, diag_bytes(g.nx, g.nk), H->stream) != cudaSuccess)
     return bail(fail(H, CHASM_ENOMEM, "device allocation failed (reductions)"));
-  e = cudaMemsetAsync(H->d_result, 0, sizeof(double) * 4, H->stream);   // the late word among them
-  if (e != cudaSuccess) return bail(cuda_fail(H, e, "reductions"));
   const size_t fbytes = (size_t)g.ncell * H->elt;
   if (!H->nuclei.empty()) {
     const int N = g.nk;
@@ -979,12 +976,9 @@ int chasm_launch_count(const chasm_handle* h, int64_t* out) {
 int chasm_sync(chasm_handle* h) {
   Handle* H = reinterpret_cast<Handle*>(h);
   if (!H) return fail(nullptr, CHASM_EINVAL, "handle is NULL");
-  int late = 0;
-  if (has_late_word(H))
-    CHASM_CUDA(H, cudaMemcpyAsync(&late, late_word(*H), sizeof(late), cudaMemcpyDeviceToHost, H->stream));
   CHASM_CUDA(H, cudaStreamSynchronize(H->stream));
   CHASM_CUDA(H, cudaGetLastError());
-  return late_status(H, late);
+  return CHASM_OK;
 }
 
 int chasm_step(chasm_handle* h, void* f, double dt, int32_t nsteps) {
@@ -1103,7 +1097,8 @@ int diag_call(chasm_handle* h, const void* f, int what, int j, double* out, size
   double* res = H->d_diag + (size_t)3 * H->g.nxp * H->g.nk;
   CHASM_CUDA(H, launch_diag(*H, f, what, j, H->d_diag, res, H->stream));
   CHASM_CUDA(H, cudaMemcpyAsync(out, res, n * sizeof(double), cudaMemcpyDeviceToHost, H->stream));
-  return chasm_sync(h);
+  CHASM_CUDA(H, cudaStreamSynchronize(H->stream));
+  return CHASM_OK;
 }
 }  // namespace
 

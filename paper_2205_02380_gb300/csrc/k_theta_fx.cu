@@ -68,7 +68,7 @@ struct FxParams {
   int nst;             // stages, 1..4
   double coef[4];      // c_s per stage
   fxc* G;              // per-CTA spectrum scratch when it is not in shared memory
-  int* late;           // set when a wait ran out (chasm_sync reports it)
+  int* late;           // set when a wait ran out (chasm_moments reports it)
 };
 
 template <int N>

@@ -1,7 +1,7 @@
 """The waits of the double-precision Coulomb kernel (csrc/group_bar.cuh) end: with a partner at
 once; without one after the given number of tries, the later waits of the block after one try, and the
 default limit after about a second (tests/c/wait_limit.cu).  The words that a wait sets when it runs out
-are what the kernel turns into NaN and the status of chasm_sync."""
+are what the kernel turns into NaN and the status of chasm_moments."""
 import os
 import subprocess
 
