@@ -6,9 +6,9 @@
 // pipe, 1.7 FMAs per clock and SM: 5.1 ms per shift at 121 x 5^2 x 32^3, 20 times the time HBM
 // needs to read and write f.  A thread transforms two real lines as one complex line, each line on
 // its own exponent (the passes are real operators, so the lines do not mix), multiplies by the
-// pass's spectrum and transforms back: three shifts 16.2 -> 2.46 ms (HBM alone 0.7).  Now two warps per
+// pass's spectrum and transforms back: three shifts 16.2 -> 2.36 ms (HBM alone 0.7).  Now two warps per
 // scheduler (254 registers) wait for their own results (2.5 warps per issue), with the FP64 pipe, which
-// converts back, 65 % busy and the integer pipe 35 %; the pass along k3 (50 % and 26 %) waits for shared
+// converts back, 68 % busy and the integer pipe 37 %; the pass along k3 (51 % and 26 %) waits for shared
 // memory as well.
 //
 // Errors: 57 bits below a line's largest entry on entry, about 3 units of the last one from each

@@ -10,15 +10,15 @@
 //
 // Bound.  The FP64 pipe (1.7 FMAs per clock and SM, measured) held the FP64 form of this kernel at
 // 94 % of what its 6.7e6 FP64 instructions per x point and stage allow at N_k = 32.  The integer
-// form issues 1.04e6 warp instructions per x point and stage (N_k = 16: 1.20e5), which at four per
-// clock and SM would take 13.6 ms at 16^3 x 32^3 (5.3 ms at 24^3 x 16^3); it issues in 40 % (48 %) of
-// the cycles, with the integer pipe at 39 % (45 %) and the multipliers at 35 % (40 %) (ncu).  At
+// form issues 1.00e6 warp instructions per x point and stage (N_k = 16: 1.15e5), which at four per
+// clock and SM would take 13.0 ms at 16^3 x 32^3 (5.1 ms at 24^3 x 16^3); it issues in 39 % (47 %) of
+// the cycles, with the integer pipe at 39 % (45 %) and the multipliers at 32 % (36 %) (ncu).  At
 // N_k = 32 64-bit vectors of 32 complex values leave registers for two warps per scheduler, which
-// wait for their own results (1.22 warps per issue), for the L2-resident spectrum and the symbol
-// (0.63), for instructions (0.51) and for shared memory (0.45).  At N_k = 16 eight groups fit (all
+// wait for their own results (1.24 warps per issue), for the L2-resident spectrum and the symbol
+// (0.67), for shared memory (0.47) and for instructions (0.47).  At N_k = 16 eight groups fit (all
 // slabs of an x point at once; four groups: 12.3 ms below): four warps per scheduler, which wait at
-// the block's barriers between the phases (1.53), for their own results (1.29) and for the pipes
-// (1.15).  P(dt): 224.3 -> 36.8 ms at 16^3 x 32^3, 77.7 -> 11.0 ms at 24^3 x 16^3.
+// the block's barriers between the phases (1.61), for their own results (1.34) and for the pipes
+// (1.09).  P(dt): 224.3 -> 35.5 ms at 16^3 x 32^3, 77.7 -> 11.0 ms at 24^3 x 16^3.
 //
 // Errors.  A vector enters a transform with 57 bits below its largest entry and leaves it with an
 // error of about 3 units of the last of them, so each of the eight transforms of a stage adds
