@@ -218,7 +218,7 @@ struct Handle {
   // reductions
   double* d_partials = nullptr;
   double* d_result = nullptr;
-  double* d_vx = nullptr;          // V(x) per x point (FP64), then the late word
+  double* d_vx = nullptr;          // V(x) per x point (FP64)
   double* d_diag = nullptr;        // diagnostics: per-x partial sums and the result
   // host-buffer entry point
   void* d_fhost = nullptr;
@@ -233,9 +233,8 @@ struct Handle {
   size_t workspace = 0;
 };
 
-// the word behind V(x) that a kernel sets when a bounded wait in it ran out; the moments copy its eight
-// bytes behind their two results
-inline int* late_word(const Handle& H) { return reinterpret_cast<int*>(H.d_vx + H.g.nxp); }
+// the word behind the moments' two results that a kernel sets when a bounded wait in it ran out
+inline int* late_word(const Handle& H) { return reinterpret_cast<int*>(H.d_result + 2); }
 
 // FP64 lines of up to kAdvDenseMax points in one patch are advected by dense matrices
 // (k_advect.cu): doubles [n * n][nk] per dimension behind the weights and shifts in AdvectTables::dev

@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(XSums<T, N>::kThreads) k_moments(const T* __re
 }
 
 __global__ void k_moments_final(const double* __restrict__ partials, int nblocks, double cell,
-                                double kin_fac, const double* __restrict__ late, double* __restrict__ out) {
+                                double kin_fac, double* __restrict__ out) {
   __shared__ double red[3][kMomThreads];
   const int tid = threadIdx.x;
   double a = 0.0, b = 0.0, c = 0.0;
@@ -64,7 +64,6 @@ __global__ void k_moments_final(const double* __restrict__ partials, int nblocks
   if (tid == 0) {
     out[0] = red[0][0] * cell;
     out[1] = (red[1][0] * kin_fac + red[2][0]) * cell;
-    out[2] = *late;
   }
 }
 
@@ -387,7 +386,7 @@ cudaError_t launch_moments(const Handle& H, const void* f, double* partials, dou
 #undef CHASM_MOM
   const double cell = H.g.h[0] * H.g.h[1] * H.g.h[2] * H.g.dk * H.g.dk * H.g.dk;
   const double kin = H.hbar * H.hbar / (2.0 * H.m) * H.g.dk * H.g.dk;
-  k_moments_final<<<1, kMomThreads, 0, s>>>(partials, nb, cell, kin, H.d_vx + H.g.nxp, result_dev);
+  k_moments_final<<<1, kMomThreads, 0, s>>>(partials, nb, cell, kin, result_dev);
   return cudaGetLastError();
 }
 
